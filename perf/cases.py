@@ -78,8 +78,8 @@ def draw(rng):
         fp64 = rng.random() < 0.2
         side = 512 if fp64 else 2048
         case = {"family": family, "neighbours": rng.choice([4, 8]), "rows": log_int(32, side),
-                "cols": log_int(32, side), "chains": rng.choice([1, 1, 2, 3, 4, 8]), "fp64": fp64, "intercept": rng.random() < 0.4,
-                "rho": rng.choice([1.0, 1.0, 0.99])}
+                "cols": log_int(32, side), "chains": rng.choice([1, 1, 2, 3, 4, 8]), "fp64": fp64,
+                "intercept": rng.random() < 0.4, "rho": rng.choice([1.0, 1.0, 0.99])}
         n = case["rows"] * case["cols"]
         return {**case, **run_length(n * case["chains"], 150 if fp64 else 400), "per_chain": n * case["chains"] <= 8192}
     if family == "volume":
