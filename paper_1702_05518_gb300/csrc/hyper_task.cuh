@@ -118,118 +118,163 @@ __device__ __forceinline__ void part_values(const Part3 *p, int which, bool need
     }
 }
 
-// The sums of task `which` over the field's tile partials, by all 32 lanes of the calling warp,
-// in a fixed order: lane l adds partials l, l + 32, l + 64, ... in that order, then a shuffle
-// tree.  S: the S (which 0) or R (which 1) sums; A: the intercept's sums when need_a.  BATCH
-// (fields of 256 or more tiles): eight loads are issued before their additions, so a warp waits
-// for one L2 round trip per 256 partials, not per 32 (the sums are the same); for fewer partials
-// one load at a time measured faster (the draws of the 512 x 512 image: 15.3 against 15.9 us per
-// sweep with eight predicated loads in flight).  CG: the partials are loaded through L2 only (the
-// resident quad kernel reads partials that other blocks of the same launch rewrite every sweep).
+// The order in which a field's tile partials are added, the same wherever they are summed: partial
+// k belongs to row (k / 32) mod 8 and lane k mod 32; a row's lane adds its partials k, k + 256, ...
+// in that order, the lane's eight rows are added in order, then a shuffle tree adds the lanes.
+// (With at most 256 partials that is lane strides in order, then the tree.)  The rows are what
+// one warp loads together (hyper_sums) or what the warps of a block take one each
+// (hyper_wide_kernel).
+constexpr int kSumRows = 8;
+
+__device__ __forceinline__ double lane_tree(double v)
+{
+#pragma unroll
+    for (int off = 16; off >= 1; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    return v;
+}
+
+// The sums of task `which` by all 32 lanes of the calling warp.  S: the S (which 0) or R (which 1)
+// sums; A: the intercept's sums when need_a.  BATCH (fields of 256 or more tiles): eight loads
+// are issued before their additions, so a warp waits for one L2 round trip per 256 partials, not
+// per 32; for fewer partials one load at a time measured faster (the draws of the 512 x 512 image:
+// 15.3 against 15.9 us per sweep with eight predicated loads in flight).  CG: the partials are
+// loaded through L2 only (the resident quad kernel reads partials that other blocks of the same
+// launch rewrite every sweep).
 template <bool BATCH, bool CG>
 __device__ __forceinline__ void hyper_sums(const HyperArgs &a, int which, bool need_a, int chain, int32_t part0,
                                            int32_t nparts, double &S, double &A)
 {
     const int lane = threadIdx.x & 31;
     const Part3 *P = a.partials + static_cast<int64_t>(part0) * a.Cp + chain;
-    constexpr int U = 8;
-    int k = lane;
     if constexpr (BATCH) {
-        for (; k + 32 * (U - 1) < nparts; k += 32 * U) {
-            double vs[U], va[U];
+        double rs[kSumRows], ra[kSumRows];
 #pragma unroll
-            for (int j = 0; j < U; ++j)
-                part_values<CG>(P + static_cast<int64_t>(k + 32 * j) * a.Cp, which, need_a, vs[j], va[j]);
+        for (int j = 0; j < kSumRows; ++j) {
+            rs[j] = 0.0;
+            ra[j] = 0.0;
+        }
+        for (int k0 = lane; k0 < nparts; k0 += 32 * kSumRows) {
+            double vs[kSumRows], va[kSumRows];
 #pragma unroll
-            for (int j = 0; j < U; ++j) {
-                S += vs[j];
-                if (need_a) A += va[j];
+            for (int j = 0; j < kSumRows; ++j) {
+                vs[j] = 0.0;
+                va[j] = 0.0;
+                if (k0 + 32 * j < nparts)
+                    part_values<CG>(P + static_cast<int64_t>(k0 + 32 * j) * a.Cp, which, need_a, vs[j], va[j]);
+            }
+#pragma unroll
+            for (int j = 0; j < kSumRows; ++j) {
+                rs[j] += vs[j];
+                if (need_a) ra[j] += va[j];
             }
         }
+#pragma unroll
+        for (int j = 0; j < kSumRows; ++j) {
+            S += rs[j];
+            if (need_a) A += ra[j];
+        }
+    } else {  // at most 256 partials
+        for (int k = lane; k < nparts; k += 32) {
+            double v, va;
+            part_values<CG>(P + static_cast<int64_t>(k) * a.Cp, which, need_a, v, va);
+            S += v;
+            if (need_a) A += va;
+        }
     }
-    for (; k < nparts; k += 32) {
-        double v, va;
-        part_values<CG>(P + static_cast<int64_t>(k) * a.Cp, which, need_a, v, va);
-        S += v;
-        if (need_a) A += va;
-    }
-    for (int off = 16; off >= 1; off >>= 1) S += __shfl_xor_sync(0xffffffffu, S, off);
-    if (need_a)
-        for (int off = 16; off >= 1; off >>= 1) A += __shfl_xor_sync(0xffffffffu, A, off);
+    S = lane_tree(S);
+    if (need_a) A = lane_tree(A);
 }
 
-// The sums of hyper_sums<*, true> from a copy of the partials laid out by field: sv[k] is the
+// The sums of hyper_sums from a copy of at most 256 partials laid out by field: sv[k] is the
 // S (which 0) or R (which 1) value of partial k and av[k] its A value, so a warp's loads cover
 // consecutive doubles (the partial records put 32 lanes' loads in 32 sectors).  Each lane issues
-// up to eight loads through L2 before adding them, in the order of hyper_sums (lane l: partials
-// l, l + 32, ...; the same shuffle tree), so the sums are bit for bit those of hyper_sums.
+// its (up to eight) loads through L2 before adding them in order, so the sums are bit for bit
+// those of hyper_sums.
 __device__ __forceinline__ void hyper_sums_by_field(const double *sv, const double *av, bool need_a,
                                                     int32_t nparts, double &S, double &A)
 {
     const int lane = threadIdx.x & 31;
-    constexpr int U = 8;
-    for (int k0 = lane; k0 < nparts; k0 += 32 * U) {
-        double vs[U], va[U];
+    double vs[kSumRows], va[kSumRows];
 #pragma unroll
-        for (int j = 0; j < U; ++j) {
-            const int k = k0 + 32 * j;
-            vs[j] = k < nparts ? __ldcg(sv + k) : 0.0;
-            va[j] = (need_a && k < nparts) ? __ldcg(av + k) : 0.0;
-        }
+    for (int j = 0; j < kSumRows; ++j) {
+        const int k = lane + 32 * j;
+        vs[j] = k < nparts ? __ldcg(sv + k) : 0.0;
+        va[j] = (need_a && k < nparts) ? __ldcg(av + k) : 0.0;
+    }
 #pragma unroll
-        for (int j = 0; j < U; ++j) {
-            if (k0 + 32 * j < nparts) {
-                S += vs[j];
-                if (need_a) A += va[j];
-            }
+    for (int j = 0; j < kSumRows; ++j) {
+        if (lane + 32 * j < nparts) {
+            S += vs[j];
+            if (need_a) A += va[j];
         }
     }
-    for (int off = 16; off >= 1; off >>= 1) S += __shfl_xor_sync(0xffffffffu, S, off);
-    if (need_a)
-        for (int off = 16; off >= 1; off >>= 1) A += __shfl_xor_sync(0xffffffffu, A, off);
+    S = lane_tree(S);
+    if (need_a) A = lane_tree(A);
 }
 
-// One task, run by all 32 lanes of the calling warp; `sweep` is the sweep being finished.
-template <typename T, bool BATCH>
+// What lane 0 needs for one task, loaded before the sums so that its latency overlaps theirs.
+struct HyperCtx {
+    int which, fi, chain;  // which: 0 tau, 1 beta0 and sigma^2
+    int64_t hc;
+    double cur, s2old, b, gpv, zb;
+    long long extra;
+    uint32_t fstream;
+    int32_t fn, frank;
+    bool pre, need_sum, need_a;
+};
+
+template <typename T>
+__device__ __forceinline__ HyperCtx hyper_ctx(const HyperArgs &a, int task, long long sweep, bool draws)
+{
+    HyperCtx c{};
+    const int pidx = task >> 1;
+    c.which = task & 1;
+    c.fi = pidx / a.Cp;
+    c.chain = pidx - c.fi * a.Cp;
+    c.hc = static_cast<int64_t>(c.fi) * a.Cp + c.chain;
+    const T *hyp = static_cast<const T *>(a.hyp);
+    long long kb = -1, bcount = 0;
+    if (draws) {
+        c.cur = c.which ? a.sig2[c.hc] : a.tau[c.hc];
+        c.s2old = a.sig2[c.hc];
+        c.b = static_cast<double>(hyp[c.hc * kHypStride + 2]);
+        c.extra = a.ctl->extra;
+        kb = sweep - a.ctl->batch_base;
+        bcount = a.ctl->batch_count;
+        c.fstream = a.fields[c.fi].stream;
+        c.fn = a.fields[c.fi].n;
+        c.frank = a.fields[c.fi].rank;
+    }
+    c.pre = a.end_of_sweep && a.gpre && kb >= 0 && kb < bcount;
+    if (draws && c.pre) {
+        const double *gp = a.gpre + (kb * a.nfields * a.Cp + pidx) * 4;
+        c.gpv = gp[c.which];
+        c.zb = gp[2];
+    }
+    c.need_sum = c.which ? (a.draw || a.draw_beta) : a.draw;
+    c.need_a = c.which && a.draw_beta;
+    return c;
+}
+
+template <typename T>
+__device__ __forceinline__ void hyper_finish(const HyperArgs &a, const HyperCtx &c, long long sweep, double S, double A)
+{
+    double val, bval;
+    hyper_draw<T>(a, c.which, c.chain, c.hc, sweep, S, A, c.cur, c.s2old, c.b, c.gpv, c.zb, c.pre, c.extra, c.fstream,
+                  c.fn, c.frank, val, bval);
+}
+
+// One task, run by all 32 lanes of the calling warp; `sweep` is the sweep being finished (fields
+// of fewer than 256 tiles).
+template <typename T>
 __device__ __forceinline__ void hyper_task(const HyperArgs &a, int task, long long sweep)
 {
     const int lane = threadIdx.x & 31;
-    const int pidx = task >> 1, which = task & 1;  // which: 0 tau, 1 beta0 and sigma^2
-    const int fi = pidx / a.Cp, chain = pidx - fi * a.Cp;
-    const int64_t hc = static_cast<int64_t>(fi) * a.Cp + chain;
-    const int32_t part0 = a.fields[fi].part0, nparts = a.fields[fi].nparts;
-    // Loads of lane 0 first, so their latency overlaps the partial sums.
-    T *hyp = static_cast<T *>(a.hyp);
-    double cur = 0.0, s2old = 0.0, b = 0.0, gpv = 0.0, zb = 0.0;
-    long long extra = 0, kb = -1, bcount = 0;
-    uint32_t fstream = 0;
-    int32_t fn = 0, frank = 0;
-    if (lane == 0) {
-        cur = which ? a.sig2[hc] : a.tau[hc];
-        s2old = a.sig2[hc];
-        b = static_cast<double>(hyp[hc * kHypStride + 2]);
-        extra = a.ctl->extra;
-        kb = sweep - a.ctl->batch_base;
-        bcount = a.ctl->batch_count;
-        fstream = a.fields[fi].stream;
-        fn = a.fields[fi].n;
-        frank = a.fields[fi].rank;
-    }
-    const bool pre = a.end_of_sweep && a.gpre && kb >= 0 && kb < bcount;
-    if (lane == 0 && pre) {
-        const double *gp = a.gpre + (kb * a.nfields * a.Cp + pidx) * 4;
-        gpv = gp[which];
-        zb = gp[2];
-    }
-    const bool need_sum = which ? (a.draw || a.draw_beta) : a.draw;
-    const bool need_a = which && a.draw_beta;
+    const HyperCtx c = hyper_ctx<T>(a, task, sweep, lane == 0);
     double S = 0.0, A = 0.0;
-    if (need_sum) hyper_sums<BATCH, false>(a, which, need_a, chain, part0, nparts, S, A);
-    if (lane == 0) {
-        double val, bval;
-        hyper_draw<T>(a, which, chain, hc, sweep, S, A, cur, s2old, b, gpv, zb, pre, extra, fstream, fn, frank, val,
-                      bval);
-    }
+    if (c.need_sum)
+        hyper_sums<false, false>(a, c.which, c.need_a, c.chain, a.fields[c.fi].part0, a.fields[c.fi].nparts, S, A);
+    if (lane == 0) hyper_finish<T>(a, c, sweep, S, A);
 }
 
 // The counters after every task of a launch has read them (one thread): the sweep number and

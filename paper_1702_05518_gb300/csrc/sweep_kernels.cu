@@ -454,21 +454,13 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? (KIND == kCsr ? 2 : 3
     }
 }
 
-// The hyperparameter stage: one warp per task of hyper_task (eight per block).  With a single
-// block its thread 0 advances the counters after a barrier; with several, the last block to
-// finish does (ticket counter; no block waits for another).
+// The hyperparameter stage for fields of fewer than 256 tiles: one warp per task of hyper_task
+// (eight per block).  With a single block its thread 0 advances the counters after a barrier; with
+// several, the last block to finish does (ticket counter; no block waits for another).
 constexpr int kHyperWarps = 8;
 
-template <typename T, bool BATCH>
-__global__ void __launch_bounds__(kHyperWarps * 32) hyper_kernel(const HyperArgs a)
+__device__ __forceinline__ void hyper_end(const HyperArgs &a, long long sweep)
 {
-    // Let the next sweep kernel be scheduled now: it does its own early work (observations,
-    // predicted normals) while this draw waits for and runs after the current sweep.
-    pdl_release();
-    pdl_wait();
-    const int task = blockIdx.x * kHyperWarps + (threadIdx.x >> 5);
-    const long long sweep = a.ctl->sweep;
-    if (task < a.nfields * a.Cp * 2) hyper_task<T, BATCH>(a, task, sweep);
     bool last = gridDim.x == 1;
     __syncthreads();
     if (!last && threadIdx.x == 0) {
@@ -479,6 +471,74 @@ __global__ void __launch_bounds__(kHyperWarps * 32) hyper_kernel(const HyperArgs
         hyper_advance(a, sweep);
         a.ctl->ticket = 0;
     }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kHyperWarps * 32) hyper_kernel(const HyperArgs a)
+{
+    // Let the next sweep kernel be scheduled now: it does its own early work (observations,
+    // predicted normals) while this draw waits for and runs after the current sweep.
+    pdl_release();
+    pdl_wait();
+    const int task = blockIdx.x * kHyperWarps + (threadIdx.x >> 5);
+    const long long sweep = a.ctl->sweep;
+    if (task < a.nfields * a.Cp * 2) hyper_task<T>(a, task, sweep);
+    hyper_end(a, sweep);
+}
+
+// The same for fields of 256 tiles or more: one block per task, its warps taking a row of the
+// partials each (the order of hyper_sums).  A launch is bound by latency: one warp per task waits
+// for an L2 round trip and eight dependent FP64 additions per 256 partials; with a block per task
+// every partial of up to 256 is loaded at once: 1222 partials of 4
+// chains 19.1 -> 9.6 us, 1240 of one chain 15.1 -> 9.2 us, 608 of 8 chains 13.4 -> 7.1 us (alone,
+// cold).
+template <typename T>
+__global__ void __launch_bounds__(kSumRows * 32) hyper_wide_kernel(const HyperArgs a)
+{
+    __shared__ double rs[kSumRows][32], ra[kSumRows][32];
+    pdl_release();
+    pdl_wait();
+    const long long sweep = a.ctl->sweep;
+    const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;
+    const HyperCtx c = hyper_ctx<T>(a, blockIdx.x, sweep, threadIdx.x == 0);
+    double S = 0.0, A = 0.0;
+    if (c.need_sum) {
+        const int nparts = a.fields[c.fi].nparts;
+        const Part3 *P = a.partials + static_cast<int64_t>(a.fields[c.fi].part0) * a.Cp + c.chain;
+        constexpr int U = 4;  // loads in flight per thread
+        for (int k0 = threadIdx.x; k0 < nparts; k0 += U * kSumRows * 32) {
+            double vs[U], va[U];
+#pragma unroll
+            for (int j = 0; j < U; ++j) {
+                const int k = k0 + j * kSumRows * 32;
+                vs[j] = 0.0;
+                va[j] = 0.0;
+                if (k < nparts)
+                    part_values<false>(P + static_cast<int64_t>(k) * a.Cp, c.which, c.need_a, vs[j], va[j]);
+            }
+#pragma unroll
+            for (int j = 0; j < U; ++j) {
+                S += vs[j];
+                if (c.need_a) A += va[j];
+            }
+        }
+        rs[row][lane] = S;
+        ra[row][lane] = A;
+        __syncthreads();
+        if (row == 0) {
+            S = 0.0;
+            A = 0.0;
+#pragma unroll
+            for (int j = 0; j < kSumRows; ++j) {
+                S += rs[j][lane];
+                if (c.need_a) A += ra[j][lane];
+            }
+            S = lane_tree(S);
+            if (c.need_a) A = lane_tree(A);
+        }
+    }
+    if (threadIdx.x == 0) hyper_finish<T>(a, c, sweep, S, A);
+    hyper_end(a, sweep);
 }
 
 // The Polya-Gamma stage of the binomial model: one warp per (slot, chain).  The slot's natural
@@ -702,13 +762,14 @@ cudaError_t launch_colour_step(int precision, int V, int kind, const StepArgs &a
 
 cudaError_t launch_hyper(int precision, const HyperArgs &a, cudaStream_t stream)
 {
-    const int grid = (a.nfields * a.Cp * 2 + kHyperWarps - 1) / kHyperWarps;
-    if (a.max_parts >= 256) {  // batched partial-sum loads (fields of many tiles)
-        if (precision == 0) return launch_sweep_kernel(hyper_kernel<float, true>, grid, kHyperWarps * 32, 0, stream, a);
-        return launch_sweep_kernel(hyper_kernel<double, true>, grid, kHyperWarps * 32, 0, stream, a);
+    if (a.max_parts >= 32 * kSumRows) {
+        const int tasks = a.nfields * a.Cp * 2;
+        if (precision == 0) return launch_sweep_kernel(hyper_wide_kernel<float>, tasks, kSumRows * 32, 0, stream, a);
+        return launch_sweep_kernel(hyper_wide_kernel<double>, tasks, kSumRows * 32, 0, stream, a);
     }
-    if (precision == 0) return launch_sweep_kernel(hyper_kernel<float, false>, grid, kHyperWarps * 32, 0, stream, a);
-    return launch_sweep_kernel(hyper_kernel<double, false>, grid, kHyperWarps * 32, 0, stream, a);
+    const int grid = (a.nfields * a.Cp * 2 + kHyperWarps - 1) / kHyperWarps;
+    if (precision == 0) return launch_sweep_kernel(hyper_kernel<float>, grid, kHyperWarps * 32, 0, stream, a);
+    return launch_sweep_kernel(hyper_kernel<double>, grid, kHyperWarps * 32, 0, stream, a);
 }
 
 cudaError_t launch_pack(int precision, const FieldDev *fields_dev, const FieldDev &f, int32_t fidx, int32_t C,
