@@ -381,21 +381,19 @@ template <> struct Vec<double, 2> {
 //   2-D 4-neighbour and 3-D 6-neighbour: colour c = parity of the coordinate sum; sub-array
 //   row = (l*H + i), column h = j / 2 (the colour-c sites of a row are j = 2h + ((c+l+i) & 1)).
 //   2-D 8-neighbour: colour c = 2 (i & 1) + (j & 1); sub-array (i / 2, j / 2).
+// (Sites and slots of a field are below 2^31: 32-bit divisions.)
 __device__ __forceinline__ int64_t lattice_slot_of_site(const FieldDev &f, int64_t site)
 {
+    const uint32_t s = static_cast<uint32_t>(site), W = static_cast<uint32_t>(f.kind == kLat3D6 ? f.dims[2] : f.dims[1]);
+    const uint32_t r = s / W, j = s - r * W;  // r = l*H + i
     if (f.kind == kLat2D8) {
-        const int64_t W = f.dims[1];
-        const int64_t i = site / W, j = site - i * W;
-        const int64_t c = 2 * (i & 1) + (j & 1);
-        return (c * f.rows + (i >> 1)) * f.cols + (j >> 1);
+        const int64_t c = 2 * (r & 1) + (j & 1);
+        return (c * f.rows + (r >> 1)) * f.cols + (j >> 1);
     }
-    const int64_t W = (f.kind == kLat3D6) ? f.dims[2] : f.dims[1];
-    const int64_t r = site / W, j = site - r * W;  // r = l*H + i
-    int64_t par = r + j;
+    uint32_t par = r + j;
     if (f.kind == kLat3D6) {
-        const int64_t H = f.dims[1];
-        const int64_t l = r / H, i = r - l * H;
-        par = l + i + j;
+        const uint32_t H = static_cast<uint32_t>(f.dims[1]);
+        par = r / H + r % H + j;
     }
     const int64_t c = par & 1;
     return (c * f.rows + r) * f.cols + (j >> 1);

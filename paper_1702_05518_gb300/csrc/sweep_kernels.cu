@@ -20,6 +20,8 @@
 // running mean and M2 of the site are updated in the same pass.
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "gmrf_device.cuh"
 #include "gmrf_internal.h"
 #include "gamma_pre.cuh"
@@ -652,29 +654,81 @@ __global__ void unpack_kernel(const FieldDev *fields, int32_t fidx, int32_t Cp, 
     }
 }
 
+// a / d for the divisor d that a launch shares (r = 1 / d): a quotient estimate and one residual
+// correction (Markstein, IBM J. Res. Dev. 1990), three FP64 operations where a division takes an
+// order of magnitude more of the FP64 pipe; quotients that are not finite take the division.
+struct Divisor {
+    double d, r;
+};
+__device__ __forceinline__ double divide(double a, const Divisor &v)
+{
+    const double q = a * v.r;
+    return isfinite(q) ? fma(fma(-q, v.d, a), v.r, q) : a / v.d;
+}
+
 // Running moments pooled over the C chains of one field, natural order, FP64: mean = the chains'
 // means averaged; var = the sum over chains of M2_c + k (mean_c - mean)^2, over C k - 1 (the
-// variance of all C k draws).  k >= 1 accumulated draws per chain.
-template <typename T>
-__global__ void pool_kernel(const FieldDev *fields, int32_t fidx, int32_t Cp, int32_t C, int64_t k, const T *mean,
-                            const T *m2, const int32_t *perm_inv, double *out_mean, double *out_var)
+// variance of all C k draws).  k >= 1 accumulated draws per chain.  CP: the layout's chains when
+// 1, 2, 4 or 8 (a site's values are loaded as vectors and kept in registers), else 0.
+//
+// Bound by the FP64 pipe (measured: about one lane per clock and SM): four FP64 operations per
+// chain and site (the mean's sum, the difference, its square, M2's sum) and three per quotient; divisions, a second pass over the means and k inside the sum
+template <typename T, int CP>
+__global__ void __launch_bounds__(256) pool_kernel(const FieldDev *fields, int32_t fidx, int32_t Cp_, int32_t C,
+                                                   int64_t k, const T *mean, const T *m2, const int32_t *perm_inv,
+                                                   double *out_mean, double *out_var)
 {
     const FieldDev f = fields[fidx];
+    const int Cp = CP ? CP : Cp_;
+    constexpr int V = CP == 0 ? 1 : (sizeof(T) == 8 ? (CP < 2 ? CP : 2) : (CP < 4 ? CP : 4));
+    constexpr int NR = CP ? CP : 1;
+    const double kd = static_cast<double>(k);
+    const Divisor by_c{static_cast<double>(C), 1.0 / static_cast<double>(C)};
+    const double dof = static_cast<double>(C * k - 1);
+    const Divisor by_dof{dof, 1.0 / dof};
     for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < f.n;
          i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
         const int64_t slot = f.slot0 + (f.kind == kCsr ? perm_inv[f.csr0 + i] : lattice_slot_of_site(f, i));
-        double mu = 0.0;
-        for (int c = 0; c < C; ++c) mu += static_cast<double>(mean[slot * Cp + c]);
-        mu /= static_cast<double>(C);
-        if (out_mean) out_mean[i] = mu;
-        if (out_var) {
-            double ss = 0.0;
-            for (int c = 0; c < C; ++c) {
-                const double d = static_cast<double>(mean[slot * Cp + c]) - mu;
-                ss += static_cast<double>(m2[slot * Cp + c]) + static_cast<double>(k) * d * d;
+        const T *mp = mean + slot * Cp, *qp = m2 + slot * Cp;
+        T mr[NR], qr[NR];
+        if constexpr (CP > 0) {
+#pragma unroll
+            for (int c = 0; c < CP; c += V) Vec<T, V>::ld(mp + c, reinterpret_cast<T(&)[V]>(mr[c]));
+            if (out_var) {
+#pragma unroll
+                for (int c = 0; c < CP; c += V) Vec<T, V>::ld(qp + c, reinterpret_cast<T(&)[V]>(qr[c]));
             }
-            out_var[i] = ss / static_cast<double>(C * k - 1);
         }
+        double mu = 0.0, ss = 0.0, dd = 0.0;
+        if constexpr (CP > 0) {
+            double md[NR];
+#pragma unroll
+            for (int c = 0; c < CP; ++c) {
+                md[c] = static_cast<double>(mr[c]);
+                if (c < C) mu += md[c];
+            }
+            if (CP > 1) mu = divide(mu, by_c);
+            if (out_var) {
+#pragma unroll
+                for (int c = 0; c < CP; ++c)
+                    if (c < C) {
+                        const double d = md[c] - mu;
+                        if (CP > 1) dd = fma(d, d, dd);
+                        ss += static_cast<double>(qr[c]);
+                    }
+            }
+        } else {
+            for (int c = 0; c < C; ++c) mu += static_cast<double>(mp[c]);
+            mu = divide(mu, by_c);
+            if (out_var)
+                for (int c = 0; c < C; ++c) {
+                    const double d = static_cast<double>(mp[c]) - mu;
+                    dd = fma(d, d, dd);
+                    ss += static_cast<double>(qp[c]);
+                }
+        }
+        if (out_mean) out_mean[i] = mu;
+        if (out_var) out_var[i] = divide(fma(kd, dd, ss), by_dof);
     }
 }
 
@@ -859,12 +913,21 @@ cudaError_t launch_pool(int precision, const FieldDev *fields_dev, const FieldDe
                         double *out_mean, double *out_var, cudaStream_t stream)
 {
     const int grid = grid_for(f.n, 256);
-    if (precision == 0)
-        pool_kernel<float><<<grid, 256, 0, stream>>>(fields_dev, fidx, Cp, C, k, static_cast<const float *>(mean),
-                                                     static_cast<const float *>(m2), perm_inv, out_mean, out_var);
-    else
-        pool_kernel<double><<<grid, 256, 0, stream>>>(fields_dev, fidx, Cp, C, k, static_cast<const double *>(mean),
-                                                      static_cast<const double *>(m2), perm_inv, out_mean, out_var);
+    auto go = [&](auto *kernel, auto *me, auto *q) {
+        kernel<<<grid, 256, 0, stream>>>(fields_dev, fidx, Cp, C, k, me, q, perm_inv, out_mean, out_var);
+    };
+    auto pick = [&](auto *me, auto *q) {
+        using T = std::remove_cv_t<std::remove_pointer_t<decltype(me)>>;
+        switch (Cp) {
+        case 1: return go(pool_kernel<T, 1>, me, q);
+        case 2: return go(pool_kernel<T, 2>, me, q);
+        case 4: return go(pool_kernel<T, 4>, me, q);
+        case 8: return go(pool_kernel<T, 8>, me, q);
+        default: return go(pool_kernel<T, 0>, me, q);
+        }
+    };
+    if (precision == 0) pick(static_cast<const float *>(mean), static_cast<const float *>(m2));
+    else pick(static_cast<const double *>(mean), static_cast<const double *>(m2));
     return cudaGetLastError();
 }
 
