@@ -187,7 +187,11 @@ typedef struct {
  * one cooperative launch, a block per tile keeping it in shared memory, a grid barrier (bounded
  * wait) per sweep, results bit for bit those of the per-sweep launches -- the quad kernel's tiles
  * for single-chain 8-neighbour fields (1024 x 1024 takes 144 blocks), else the fused sweep's when
- * every thread holds all chains (1, 2 or 4 in the layout).  On by default in FP32;
+ * every thread holds all chains (1, 2 or 4 in the layout).  An FP32 sampler of a single graph beyond
+ * the small ones (weighted edges, more sites, neighbours or sites per class) and of up to 8 chains
+ * runs its colour steps in one cooperative launch per batch of sweeps as well, with a grid barrier
+ * per colour step (results equal up to rounding; its state stays in device memory, and
+ * gmrf_info.resident stays 0), unless a tuning of the colour-step kernels is given.  On by default in FP32;
  * GMRF_FLAG_RESIDENT asks for the small-lattice form in FP64 as well, GMRF_FLAG_NO_RESIDENT keeps
  * the per-sweep launches.
  * gmrf_info.resident tells which path a sampler took. */
@@ -197,7 +201,7 @@ typedef struct {
 /* GMRF_FLAG_TEST_STALL (for tests of failure handling only): on the resident graph path with a
  * cluster of two or more blocks per chain (a single graph of 4096 or more sites), every colour
  * step of the cluster kernel expects 16 more bytes than the other blocks send, and on the resident
- * tile paths every grid barrier expects one arrival more than there are blocks, so the bounded
+ * tile paths and the grid sweeps every grid barrier expects one arrival more than there are blocks, so the bounded
  * wait gives up (after 1 ms with this flag, instead of 1 s), as a lost exchange would make it; the
  * kernel still finishes, and the next call that reads the counters returns GMRF_E_TIMEOUT. */
 #define GMRF_FLAG_TEST_STALL 8

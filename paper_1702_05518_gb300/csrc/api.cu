@@ -224,9 +224,11 @@ struct gmrf_sampler {
     int res_cluster = 1, res_own_max = 0;                      // graph: blocks per chain, their share
     int res_positions = 0;                                     // graph: 1 = one position per thread
     int32_t res_SR = 0, res_SC = 0;
+    int grid_blocks = 0;  // grid sweeps (colour_grid.cu): blocks of the launch, 0 not used
     size_t res_smem = 0;
     void *res_z = nullptr;  // [res_batch][C][colours][NI][site threads] normals of a batch
-    double *res_pm = nullptr;  // fused resident tiles, Cp = 4: the tile partials by field (TileResArgs)
+    double *res_pm = nullptr;  // fused resident tiles, Cp = 4: the tile partials by field (TileResArgs);
+                               // grid sweeps: the blocks' (GridSweepArgs)
 
     cudaError_t alloc(void **p, size_t b)
     {
@@ -646,6 +648,24 @@ cudaError_t plan_tile_resident(gmrf_sampler *s)
     return cudaSuccess;
 }
 
+// Grid sweeps (colour_grid.cu) for a single FP32 graph that has no resident form (weighted edges,
+// 32768 sites or more, more than 16 neighbours, large classes): its colour steps are bound by
+// latency, and a launch each costs more than a grid barrier.  A tuning of the colour-step kernels
+// asks for those kernels.
+cudaError_t plan_grid(gmrf_sampler *s, const std::vector<int32_t> &coff0)
+{
+    if (s->precision != GMRF_FP32 || s->tune.step_tile || s->tune.chains_per_thread || s->tune.graph_cluster)
+        return cudaSuccess;
+    const HostField &h = s->hf[0];
+    if (h.kind != GMRF_CSR || coff0.size() != size_t(h.ncolors) + 1) return cudaSuccess;
+    int largest = 0;
+    for (int c = 0; c < h.ncolors; ++c) largest = std::max(largest, coff0[c + 1] - coff0[c]);
+    cudaError_t e = plan_csr_grid(s->Cp, s->w != nullptr, h.ncolors, largest, &s->grid_blocks);
+    if (e != cudaSuccess || !s->grid_blocks) return e;
+    s->res_batch = std::min(128, std::max(64, s->opts.graph_sweeps));
+    return s->alloc_t(&s->res_pm, static_cast<size_t>(3) * s->Cp * s->grid_blocks, sizeof(double));
+}
+
 // The resident path applies to a single fused 2-D lattice field with the Gaussian likelihood whose
 // chain fits in shared memory (state, observations, mean and M2 with a ring of zeros: cells below
 // 2^16, sites below 2^16) and whose colour classes have at most 2 x 576 (8-neighbour) or 4 x 576
@@ -667,7 +687,7 @@ cudaError_t plan_resident(gmrf_sampler *s, const std::vector<int32_t> &coff0)
         // within the site threads' positions, and state, mean and M2 in shared memory.
         const HostField &h = s->hf[0];
         if (h.weighted || f.n >= 32768 || h.max_degree > 16 || h.ncolors > 64 || coff0.size() != size_t(h.ncolors) + 1)
-            return cudaSuccess;
+            return plan_grid(s, coff0);
         // A cluster of CL blocks per chain (at most 152 blocks in all): one block per 2048 sites.
         int cl = 1;
         while (cl < 8 && f.n >= 2048 * 2 * cl && s->C * 2 * cl <= 152) cl *= 2;
@@ -675,12 +695,12 @@ cudaError_t plan_resident(gmrf_sampler *s, const std::vector<int32_t> &coff0)
         int own_max = 0, share_max = 0;
         for (int c = 0; c < h.ncolors; ++c) {
             const int len = coff0[c + 1] - coff0[c], q = (len + cl - 1) / cl;
-            if (q > csr_resident_max_positions()) return cudaSuccess;
+            if (q > csr_resident_max_positions()) return plan_grid(s, coff0);
             own_max += q;
             share_max = std::max(share_max, q);
         }
         const size_t smem = (static_cast<size_t>(f.n) + 1 + 2 * static_cast<size_t>(own_max)) * tsize(s->precision);
-        if (smem > 220 * 1024) return cudaSuccess;
+        if (smem > 220 * 1024) return plan_grid(s, coff0);
         cudaError_t e = prepare_csr_resident(s->precision, smem);
         if (e == cudaSuccess) e = s->alloc_t(&s->res_nbr, static_cast<size_t>(f.n), sizeof(uint4));
         if (e == cudaSuccess) e = s->alloc_t(&s->res_nbr2, static_cast<size_t>(f.n), sizeof(uint4));
@@ -850,6 +870,18 @@ TileResArgs tile_resident_args(gmrf_sampler *s, int count, int draw, int draw_be
     return r;
 }
 
+GridSweepArgs grid_args(gmrf_sampler *s, int count, int draw, int draw_beta)
+{
+    GridSweepArgs g{};
+    g.s = step_args(s, 0, s->fd[0].kind, 1);
+    g.h = hyper_args(s, draw, draw_beta, 1);
+    g.count = count;
+    g.pm = s->res_pm;
+    g.extra_arrivals = s->test_stall ? 1u : 0u;
+    g.wait_ns = s->test_stall ? 1000000ull : kWaitNs;
+    return g;
+}
+
 // One stage of a sweep (see gmrf_launch_stage); `draw`, `draw_beta` and `end_of_sweep` only
 // matter for the hyperparameter stage.
 // Description of stage k of a sweep (also its NVTX range name).
@@ -919,6 +951,16 @@ cudaError_t enqueue_sweeps(gmrf_sampler *s, int nsweeps, int with_hyper, cudaStr
     cudaError_t e = cudaSuccess;
     const int draw = (with_hyper && !s->model.fix_hyper) ? 1 : 0;
     const int draw_beta = (with_hyper && has_beta(s)) ? 1 : 0;
+    if (s->grid_blocks) {
+        for (int k = 0; k < nsweeps && e == cudaSuccess;) {
+            const NvtxRange range("grid sweeps");
+            const int cnt = std::min(s->res_batch, nsweeps - k);
+            if (draw || draw_beta) e = launch_pre(s, cnt, st);
+            if (e == cudaSuccess) e = launch_csr_grid(s->grid_blocks, grid_args(s, cnt, draw, draw_beta), st);
+            k += cnt;
+        }
+        return e;
+    }
     if (s->resident) {
         // Batches of sweeps: the batch's unit-rate Gamma variates and normals, then all its sweeps
         // in one launch.

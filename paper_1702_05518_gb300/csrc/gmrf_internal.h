@@ -333,6 +333,24 @@ cudaError_t launch_lattice_fused_resident(int kind, int threads, int Cp, const T
 cudaError_t launch_lattice_quad_resident(int qcs, int nt, int nq, const TileResArgs &ra, size_t smem,
                                          cudaStream_t stream);
 
+// Grid sweeps (colour_grid.cu): a batch of whole sweeps of a single FP32 field's colour steps in one
+// cooperative launch, a grid barrier per colour step.
+struct GridSweepArgs {
+    StepArgs s;               // the field's buffers (update 1; tiles unused)
+    HyperArgs h;              // the conjugate draws at the end of each sweep (end_of_sweep 1)
+    int32_t count;            // sweeps of the launch
+    double *pm;               // [Cp][S, R, A][block] the blocks' partial sums
+    uint32_t extra_arrivals;  // 0; 1 under GMRF_FLAG_TEST_STALL (no grid barrier completes)
+    uint64_t wait_ns;         // limit of a wait at the grid barrier
+};
+// A block's items (a position's chain vector of up to 4) of the largest colour class: at most
+// kGridItems per thread (beyond, a launch per colour keeps the chip as full and costs nothing
+// beside its work), and at least kGridMinItems (fewer blocks make a cheaper barrier).
+constexpr int kGridItems = 8, kGridMinItems = 96;
+// The blocks of a graph's grid sweep, 0 where it does not apply.
+cudaError_t plan_csr_grid(int Cp, bool weighted, int ncolors, int largest_class, int *blocks);
+cudaError_t launch_csr_grid(int blocks, const GridSweepArgs &ra, cudaStream_t stream);
+
 // Jones-Plassmann colouring and colour-permuted CSR layout (csr_build.cu).
 struct CsrBuild {
     int32_t n;
