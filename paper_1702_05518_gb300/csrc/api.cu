@@ -648,19 +648,24 @@ cudaError_t plan_tile_resident(gmrf_sampler *s)
     return cudaSuccess;
 }
 
-// Grid sweeps (colour_grid.cu) for a single FP32 graph that has no resident form (weighted edges,
-// 32768 sites or more, more than 16 neighbours, large classes): its colour steps are bound by
-// latency, and a launch each costs more than a grid barrier.  A tuning of the colour-step kernels
-// asks for those kernels.
+// Grid sweeps (colour_grid.cu) for a single FP32 field whose colour steps are bound by latency, so that
+// a launch each costs more than a grid barrier: a graph that has no resident form (weighted edges,
+// 32768 sites or more, more than 16 neighbours, large classes), or a 3-D lattice whose sites'
+// normals fit the threads' registers.  A tuning of the colour-step kernels asks for those kernels.
 cudaError_t plan_grid(gmrf_sampler *s, const std::vector<int32_t> &coff0)
 {
-    if (s->precision != GMRF_FP32 || s->tune.step_tile || s->tune.chains_per_thread || s->tune.graph_cluster)
+    if (s->precision != GMRF_FP32 || s->tune.step_tile || s->tune.chains_per_thread || s->tune.graph_cluster ||
+        s->tune.wide_3d)
         return cudaSuccess;
     const HostField &h = s->hf[0];
-    if (h.kind != GMRF_CSR || coff0.size() != size_t(h.ncolors) + 1) return cudaSuccess;
-    int largest = 0;
-    for (int c = 0; c < h.ncolors; ++c) largest = std::max(largest, coff0[c + 1] - coff0[c]);
-    cudaError_t e = plan_csr_grid(s->Cp, s->w != nullptr, h.ncolors, largest, &s->grid_blocks);
+    cudaError_t e = cudaSuccess;
+    if (h.kind == GMRF_CSR && coff0.size() == size_t(h.ncolors) + 1) {
+        int largest = 0;
+        for (int c = 0; c < h.ncolors; ++c) largest = std::max(largest, coff0[c + 1] - coff0[c]);
+        e = plan_csr_grid(s->Cp, s->w != nullptr, h.ncolors, largest, &s->grid_blocks);
+    } else if (h.kind == GMRF_LATTICE3D_6) {
+        e = plan_lattice3d_grid(s->Cp, s->fd[0].rows, h.dims[2], &s->grid_blocks);
+    }
     if (e != cudaSuccess || !s->grid_blocks) return e;
     s->res_batch = std::min(128, std::max(64, s->opts.graph_sweeps));
     return s->alloc_t(&s->res_pm, static_cast<size_t>(3) * s->Cp * s->grid_blocks, sizeof(double));
@@ -722,6 +727,7 @@ cudaError_t plan_resident(gmrf_sampler *s, const std::vector<int32_t> &coff0)
         s->resident = 2;
         return cudaSuccess;
     }
+    if (f.kind == GMRF_LATTICE3D_6) return plan_grid(s, coff0);
     if (!s->hf[0].fused) return cudaSuccess;
     if (f.kind != GMRF_LATTICE2D_4 && f.kind != GMRF_LATTICE2D_8) return cudaSuccess;
     const bool e8 = f.kind == GMRF_LATTICE2D_8;
@@ -956,7 +962,10 @@ cudaError_t enqueue_sweeps(gmrf_sampler *s, int nsweeps, int with_hyper, cudaStr
             const NvtxRange range("grid sweeps");
             const int cnt = std::min(s->res_batch, nsweeps - k);
             if (draw || draw_beta) e = launch_pre(s, cnt, st);
-            if (e == cudaSuccess) e = launch_csr_grid(s->grid_blocks, grid_args(s, cnt, draw, draw_beta), st);
+            const GridSweepArgs ga = grid_args(s, cnt, draw, draw_beta);
+            if (e == cudaSuccess)
+                e = s->fd[0].kind == GMRF_CSR ? launch_csr_grid(s->grid_blocks, ga, st)
+                                              : launch_lattice3d_grid(s->grid_blocks, s->fd[0].rows, s->fd[0].dims[2], ga, st);
             k += cnt;
         }
         return e;

@@ -342,6 +342,8 @@ struct GridSweepArgs {
     double *pm;               // [Cp][S, R, A][block] the blocks' partial sums
     uint32_t extra_arrivals;  // 0; 1 under GMRF_FLAG_TEST_STALL (no grid barrier completes)
     uint64_t wait_ns;         // limit of a wait at the grid barrier
+    uint32_t u_m;             // 3-D lattices: invariant-divisor constants of the units in a row
+    int32_t u_s;              // (set by launch_lattice3d_grid)
 };
 // A block's items (a position's chain vector of up to 4) of the largest colour class: at most
 // kGridItems per thread (beyond, a launch per colour keeps the chip as full and costs nothing
@@ -350,6 +352,9 @@ constexpr int kGridItems = 8, kGridMinItems = 96;
 // The blocks of a graph's grid sweep, 0 where it does not apply.
 cudaError_t plan_csr_grid(int Cp, bool weighted, int ncolors, int largest_class, int *blocks);
 cudaError_t launch_csr_grid(int blocks, const GridSweepArgs &ra, cudaStream_t stream);
+// The same for a 3-D lattice of `rows` rows of W sites.
+cudaError_t plan_lattice3d_grid(int Cp, int64_t rows, int W, int *blocks);
+cudaError_t launch_lattice3d_grid(int blocks, int64_t rows, int W, const GridSweepArgs &ra, cudaStream_t stream);
 
 // Jones-Plassmann colouring and colour-permuted CSR layout (csr_build.cu).
 struct CsrBuild {

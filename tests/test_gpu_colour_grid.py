@@ -44,6 +44,18 @@ FIELDS = {
 }
 
 
+# Units of a thread (up to four consecutive sites) across row and plane ends of every parity, single
+# rows, columns and planes, a last unit that is not full.
+VOLUMES = [(1, 1, 1), (1, 1, 9), (7, 1, 1), (1, 6, 1), (5, 3, 2), (3, 5, 3), (3, 4, 7), (2, 3, 6), (9, 8, 5), (17, 13, 11),
+           (20, 24, 28)]
+# One, two or four units per thread: (chains, extents) at the sizes where the number grows.
+UNITS = [(1, (61, 71, 73)), (1, (89, 85, 83)), (2, (50, 61, 53)), (2, (72, 70, 67)), (4, (55, 54, 53)), (8, (44, 43, 45))]
+
+
+def _volume(dims):
+    return wl.small_lattice(wl.LATTICE3D_6, dims, 8)
+
+
 def _run(f, chains, calls, intercept=False, **kw):
     with g.Sampler([f], precision=g.FP32, chains=chains, seed=31, trace_capacity=512, intercept=intercept, **kw) as s:
         for n, hyper in calls:
@@ -61,9 +73,9 @@ KEYS = ("x", "mean", "var", "tau_trace", "sigma2_trace")
 
 
 @pytest.mark.parametrize("chains", [1, 2, 3, 8])
-@pytest.mark.parametrize("name", sorted(FIELDS))
+@pytest.mark.parametrize("name", sorted(FIELDS) + VOLUMES, ids=str)
 def test_parity_with_the_oracle(name, chains):
-    f = FIELDS[name]()
+    f = FIELDS[name]() if name in FIELDS else _volume(name)
     one, _ = _run(f, chains, [(1, True)])
     st, _ = run_oracle(f, chains, 1, seed=31, stream=0)
     assert max(relerr(one[c]["x"], st.x[c]) for c in range(chains)) <= TOL_FP32_1
@@ -81,10 +93,21 @@ def test_parity_with_the_oracle(name, chains):
             assert relerr(res[c]["beta0_trace"], out["beta0_trace"][c]) <= TOL_FP32_1000
 
 
-@pytest.mark.parametrize("name", ["delaunay_1000", "star_700"])
+@pytest.mark.parametrize("chains,dims", UNITS)
+def test_units_per_thread(chains, dims):
+    f = _volume(dims)
+    res, _ = _run(f, chains, [(3, True)], intercept=chains == 2)
+    st, out = run_oracle(f, chains, 3, seed=31, stream=0, intercept=chains == 2, burn_in=0)
+    for c in range(chains):
+        assert relerr(res[c]["x"], st.x[c]) <= TOL_FP32_1000
+        assert relerr(res[c]["mean"], st.mean[c]) <= TOL_FP32_1000
+        assert trace_relerr(res[c]["tau_trace"], out["tau_trace"][c]) <= TOL_FP32_1000
+
+
+@pytest.mark.parametrize("name", ["delaunay_1000", "star_700", (17, 13, 11)], ids=str)
 @pytest.mark.parametrize("thin", [1, 3])
 def test_any_cut_into_launches_is_the_same_bit_for_bit(name, thin):
-    f = FIELDS[name]()
+    f = FIELDS[name]() if name in FIELDS else _volume(name)
     ref, _ = _run(f, 3, [(150, True)], burn_in=20, thin=thin)
     for kw in ({"graph_sweeps": 7}, {"graph_sweeps": 128}):
         got, _ = _run(f, 3, [(1, True), (148, True), (1, True)], burn_in=20, thin=thin, **kw)
@@ -93,9 +116,9 @@ def test_any_cut_into_launches_is_the_same_bit_for_bit(name, thin):
                 assert np.array_equal(got[c][key], ref[c][key]), key
 
 
-@pytest.mark.parametrize("name", ["delaunay_1000", "delaunay_33000"])
+@pytest.mark.parametrize("name", ["delaunay_1000", "delaunay_33000", (20, 24, 28), (60, 60, 61)], ids=str)
 def test_agrees_with_a_launch_per_colour(name):
-    f = FIELDS[name]()
+    f = FIELDS[name]() if name in FIELDS else _volume(name)
     calls = [(5, True), (3, False), (12, True)]
     a, ia = _run(f, 4, calls, burn_in=4, thin=2)
     b, ib = _run(f, 4, calls, burn_in=4, thin=2, flags=g.FLAG_NO_RESIDENT)
@@ -105,8 +128,9 @@ def test_agrees_with_a_launch_per_colour(name):
             assert relerr(a[c][key], b[c][key]) <= TOL_FP32_1000, key
 
 
-def test_barrier_timeout_reports_and_poisons():
-    f = FIELDS["delaunay_1000"]()
+@pytest.mark.parametrize("name", ["delaunay_1000", (17, 13, 11)], ids=str)
+def test_barrier_timeout_reports_and_poisons(name):
+    f = FIELDS[name]() if name in FIELDS else _volume(name)
     with g.Sampler([f], precision=g.FP32, chains=2, seed=3, flags=g.FLAG_TEST_STALL) as s:
         s.sweep(10)
         with pytest.raises(g.GmrfError) as e:
