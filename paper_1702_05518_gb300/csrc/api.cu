@@ -170,6 +170,13 @@ struct gmrf_sampler {
     int32_t fQCS[4] = {0, 0, 0, 0}, fNQ[4] = {0, 0, 0, 0};
     size_t fsmem_gen[4] = {0, 0, 0, 0};  // the quad tiling's shared memory in lattice_fused_kernel
     size_t fsmem[4] = {0, 0, 0, 0};
+    // Marching warps (lattice_march.cu) for FP32 2-D lattices: rows of a chunk per kind (0: not used),
+    // blocks of a sweep, and whether a batch of sweeps runs in one cooperative launch.
+    int march_rows[4] = {0, 0, 0, 0};
+    MarchTile *mtiles_dev = nullptr;
+    int32_t mtile_off[4] = {0, 0, 0, 0}, mtile_cnt[4] = {0, 0, 0, 0};
+    bool march_grid = false;
+    int march_zrows = 0;
     FieldDev *fields_dev = nullptr;
     Tile *tiles_dev = nullptr;
     void *x = nullptr, *y = nullptr, *mean = nullptr, *m2 = nullptr;
@@ -619,6 +626,48 @@ cudaError_t launch_pre(gmrf_sampler *s, int count, cudaStream_t st)
     return launch_gamma_pre(gamma_pre_args(s, count), st);
 }
 
+// Rows of a marching warp's chunk (lattice_march.cu), by cost: waves of blocks (one per SM) times the
+// rows a warp walks, the recomputed ones and a fixed cost of a block worth four rows included.
+int march_chunk_rows(const gmrf_sampler *s, int kind)
+{
+    double best = 1e300;
+    int rows = 2;
+    const int step = kind == GMRF_LATTICE2D_8 ? 2 : 1;
+    for (int r = 2; r <= 256; r += step) {
+        int64_t blocks = 0;
+        for (auto &h : s->hf)
+            if (h.kind == kind) blocks += march_blocks(kind, s->Cp, h.dims[0], h.dims[1], r);
+        const double cost = std::ceil(static_cast<double>(blocks) / 152.0) * (r + 2.0 / step + 4.0);
+        if (cost < best * 0.999) {
+            best = cost;
+            rows = r;
+        }
+    }
+    return rows;
+}
+
+// Marching warps in place of the tiles: FP32 samplers of one or two chains, unless a tuning of the
+// tiled kernels is given or the field is the only one and its tiles fit in one wave (which then
+// stay in shared memory for a batch of sweeps, plan_tile_resident).  Where the lines lie (us per sweep,
+// marching / tiles): one wave of tiles 300 x 244, one chain 12.4 / 8.5, 512 x 512 12.7 / 9.6,
+// 1024 x 1023 18 / 17.5; beyond one wave 1500 x 1300 two chains 26 / 39 (8-neighbour 28 / 43),
+// 2047 x 1931 one chain 24 / 58.
+cudaError_t plan_march(gmrf_sampler *s, int kind)
+{
+    if (s->precision != GMRF_FP32 || s->Cp > 2 || s->tune.fused_rows[kind] || s->tune.fused_threads[kind] ||
+        (s->tune.chains_per_thread != 0 && s->tune.chains_per_thread != s->Cp))
+        return cudaSuccess;
+    if (s->nfields == 1 && s->tune.chains_per_thread == 0) {
+        const int32_t *d = s->hf[0].dims;
+        const int tiles = ((d[0] + s->fTR[kind] - 1) / s->fTR[kind]) * ((d[1] + s->fTC[kind] - 1) / s->fTC[kind]);
+        bool fits = false;
+        const cudaError_t e = lattice_fused_resident_fits(kind, s->fNT[kind], s->Cp, s->fsmem[kind], tiles, &fits);
+        if (e != cudaSuccess || fits) return e;
+    }
+    s->march_rows[kind] = march_chunk_rows(s, kind);
+    return cudaSuccess;
+}
+
 // The resident tile forms, for a single 2-D lattice field whose per-sweep kernel's tiles can all be
 // resident at once (one block each): the quad kernel's (single-chain FP32 8-neighbour fields), else
 // the fused sweep's when it runs the fast form (FP32, every thread holding all chains).
@@ -630,9 +679,36 @@ cudaError_t plan_tile_resident(gmrf_sampler *s)
     if (s->fQCS[kind]) {
         const cudaError_t e = lattice_quad_resident_fits(s->fQCS[kind], s->fNT[kind], s->fNQ[kind], s->fsmem[kind],
                                                          s->ftile_cnt[kind], &fits);
-        if (e != cudaSuccess || !fits) return e;
+        if (e != cudaSuccess) return e;
+        if (fits) {
+            s->res_batch = std::min(128, std::max(64, s->opts.graph_sweeps));
+            s->resident = 3;
+            return cudaSuccess;
+        }
+        if (s->tune.quad_config || s->tune.quad_rows) return cudaSuccess;
+    }
+    if (s->march_rows[kind] || s->fQCS[kind]) {
+        // Batches of sweeps by marching warps, also of a field whose single sweeps take the quad
+        // kernel's tiles in several waves (2048 x 2048: 26 us per sweep against 49).
+        const int rows = s->march_rows[kind] ? s->march_rows[kind] : march_chunk_rows(s, kind);
+        if (!s->march_rows[kind]) {
+            std::vector<MarchTile> mt;
+            const int nb = march_blocks(kind, s->Cp, s->hf[0].dims[0], s->hf[0].dims[1], rows);
+            for (int b = 0; b < nb; ++b) mt.push_back({0, b, rows, 0});
+            cudaError_t et = s->alloc_t(&s->mtiles_dev, mt.size(), sizeof(MarchTile));
+            if (et == cudaSuccess)
+                et = cudaMemcpy(s->mtiles_dev, mt.data(), mt.size() * sizeof(MarchTile), cudaMemcpyHostToDevice);
+            if (et != cudaSuccess) return et;
+            s->mtile_cnt[kind] = nb;
+        }
+        const int zrows = march_ahead_rows(s->Cp, rows);
+        cudaError_t em = plan_march_grid(kind, s->Cp, s->mtile_cnt[kind], zrows, &fits);
+        if (em == cudaSuccess && fits)
+            em = s->alloc_t(&s->res_pm, static_cast<size_t>(3) * s->Cp * s->mtile_cnt[kind], sizeof(double));
+        if (em != cudaSuccess || !fits) return em;
+        s->march_grid = true;
+        s->march_zrows = zrows;
         s->res_batch = std::min(128, std::max(64, s->opts.graph_sweeps));
-        s->resident = 3;
         return cudaSuccess;
     }
     if (s->precision != GMRF_FP32 || s->V != s->Cp || (s->Cp != 1 && s->Cp != 2 && s->Cp != 4)) return cudaSuccess;
@@ -888,6 +964,29 @@ GridSweepArgs grid_args(gmrf_sampler *s, int count, int draw, int draw_beta)
     return g;
 }
 
+MarchArgs march_args(gmrf_sampler *s, int kind, int update, int accumulate)
+{
+    MarchArgs m{};
+    m.f = fused_args(s, kind, update, accumulate);
+    m.tiles = s->mtiles_dev + s->mtile_off[kind];
+    m.ntiles = s->mtile_cnt[kind];
+    m.intercept = has_beta(s) ? 1 : 0;
+    philox_round_keys(m.f.key, m.rk);
+    return m;
+}
+
+MarchArgs march_grid_args(gmrf_sampler *s, int count, int draw, int draw_beta)
+{
+    MarchArgs m = march_args(s, s->fd[0].kind, 1, 1);
+    m.h = hyper_args(s, draw, draw_beta, 1);
+    m.count = count;
+    m.zrows = s->march_zrows;
+    m.pm = s->res_pm;
+    m.extra_arrivals = s->test_stall ? 1u : 0u;
+    m.wait_ns = s->test_stall ? 1000000ull : kWaitNs;
+    return m;
+}
+
 // One stage of a sweep (see gmrf_launch_stage); `draw`, `draw_beta` and `end_of_sweep` only
 // matter for the hyperparameter stage.
 // Description of stage k of a sweep (also its NVTX range name).
@@ -917,6 +1016,7 @@ cudaError_t enqueue_stage(gmrf_sampler *s, size_t k, int update, int accumulate,
 {
     const NvtxRange range(stage_name(s, k));
     const gmrf_sampler::Stage &g = s->stages[k];
+    if (g.type == 1 && s->march_rows[g.kind]) return launch_march(g.kind, march_args(s, g.kind, update, accumulate), st);
     if (g.type == 1) {
         FusedArgs fa = fused_args(s, g.kind, update, accumulate);
         if (s->fQCS[g.kind]) {
@@ -957,6 +1057,17 @@ cudaError_t enqueue_sweeps(gmrf_sampler *s, int nsweeps, int with_hyper, cudaStr
     cudaError_t e = cudaSuccess;
     const int draw = (with_hyper && !s->model.fix_hyper) ? 1 : 0;
     const int draw_beta = (with_hyper && has_beta(s)) ? 1 : 0;
+    if (s->march_grid) {
+        const int kd = s->fd[0].kind;
+        for (int k = 0; k < nsweeps && e == cudaSuccess;) {
+            const NvtxRange range("marching sweeps");
+            const int cnt = std::min(s->res_batch, nsweeps - k);
+            if (draw || draw_beta) e = launch_pre(s, cnt, st);
+            if (e == cudaSuccess) e = launch_march_grid(kd, march_grid_args(s, cnt, draw, draw_beta), st);
+            k += cnt;
+        }
+        return e;
+    }
     if (s->grid_blocks) {
         for (int k = 0; k < nsweeps && e == cudaSuccess;) {
             const NvtxRange range("grid sweeps");
@@ -1438,6 +1549,7 @@ gmrf_status build_chromatic(gmrf_sampler *s, const gmrf_field_desc *fields, std:
             s->fTC[kind] = tc;
             s->fsmem[kind] = lattice_fused_smem(s->precision, kind, s->Cp, tr, tc);
             CK(prepare_lattice_fused(s->precision, s->V, kind, s->fsmem[kind]));
+            CK(plan_march(s, kind));
         }
     }
     int64_t total_elems = 0;
@@ -1486,10 +1598,18 @@ gmrf_status build_chromatic(gmrf_sampler *s, const gmrf_field_desc *fields, std:
     for (auto &h : s->hf) s->kmax = std::max(s->kmax, h.ncolors);
     std::vector<std::vector<Tile>> by_colour(s->kmax);
     std::vector<TileXY> fz[4];
+    std::vector<MarchTile> mz[4], mall;
     int part = 0;
     for (int fi = 0; fi < s->nfields; ++fi) {
         FieldDev &d = s->fd[fi];
         d.part0 = part;
+        if (s->march_rows[d.kind]) {
+            s->hf[fi].fused = true;
+            const int nb = march_blocks(d.kind, s->Cp, d.dims[0], d.dims[1], s->march_rows[d.kind]);
+            for (int b = 0; b < nb; ++b) mz[d.kind].push_back({fi, b, s->march_rows[d.kind], part++});
+            d.nparts = part - d.part0;
+            continue;
+        }
         if (fused_kind[d.kind]) {
             s->hf[fi].fused = true;
             for (int i0 = 0; i0 < d.dims[0]; i0 += s->fTR[d.kind])
@@ -1553,7 +1673,10 @@ gmrf_status build_chromatic(gmrf_sampler *s, const gmrf_field_desc *fields, std:
         s->ftile_off[kind] = static_cast<int32_t>(fall.size());
         s->ftile_cnt[kind] = static_cast<int32_t>(fz[kind].size());
         fall.insert(fall.end(), fz[kind].begin(), fz[kind].end());
-        if (!fz[kind].empty()) s->stages.push_back({1, kind, -1});
+        s->mtile_off[kind] = static_cast<int32_t>(mall.size());
+        s->mtile_cnt[kind] = static_cast<int32_t>(mz[kind].size());
+        mall.insert(mall.end(), mz[kind].begin(), mz[kind].end());
+        if (!fz[kind].empty() || !mz[kind].empty()) s->stages.push_back({1, kind, -1});
     }
     std::vector<Tile> all;
     s->tile_off.assign(static_cast<size_t>(s->kmax) * 4, 0);
@@ -1577,7 +1700,7 @@ gmrf_status build_chromatic(gmrf_sampler *s, const gmrf_field_desc *fields, std:
                 ++sweep_kernels;
                 kind = st.type == 1 ? st.kind : -2;
             }
-        s->early_kind = (sweep_kernels == 1 && kind >= 0) ? kind : -1;
+        s->early_kind = (sweep_kernels == 1 && kind >= 0 && !s->march_rows[kind]) ? kind : -1;
     }
     CK(plan_resident(s, coff_host[0]));
     {
@@ -1596,7 +1719,10 @@ gmrf_status build_chromatic(gmrf_sampler *s, const gmrf_field_desc *fields, std:
     CK(s->alloc_t(&s->tiles_dev, std::max<size_t>(all.size(), 1), sizeof(Tile)));
     if (!all.empty())
         CK(cudaMemcpyAsync(s->tiles_dev, all.data(), sizeof(Tile) * all.size(), cudaMemcpyHostToDevice, s->stream));
-    if (!fall.empty()) CK(s->alloc(&s->x_alt, static_cast<size_t>(slots) * Cp * T));
+    if (!fall.empty() || !mall.empty()) CK(s->alloc(&s->x_alt, static_cast<size_t>(slots) * Cp * T));
+    if (!mall.empty()) CK(s->alloc_t(&s->mtiles_dev, mall.size(), sizeof(MarchTile)));
+    if (!mall.empty())
+        CK(cudaMemcpyAsync(s->mtiles_dev, mall.data(), sizeof(MarchTile) * mall.size(), cudaMemcpyHostToDevice, s->stream));
     CK(s->alloc_t(&s->ftiles_dev, std::max<size_t>(fall.size(), 1), sizeof(TileXY)));
     if (!fall.empty())
         CK(cudaMemcpyAsync(s->ftiles_dev, fall.data(), sizeof(TileXY) * fall.size(), cudaMemcpyHostToDevice,

@@ -356,6 +356,36 @@ cudaError_t launch_csr_grid(int blocks, const GridSweepArgs &ra, cudaStream_t st
 cudaError_t plan_lattice3d_grid(int Cp, int64_t rows, int W, int *blocks);
 cudaError_t launch_lattice3d_grid(int blocks, int64_t rows, int W, const GridSweepArgs &ra, cudaStream_t stream);
 
+// Marching warps (lattice_march.cu) for FP32 2-D lattice fields.  A block of a field runs 16 chunks
+// (strip of columns, `rows` rows, chain group); its partial sums are slot `part`.
+struct MarchTile {
+    int32_t field;
+    int32_t block;      // of the field
+    int32_t rows;       // of a chunk (even on the 8-neighbour lattice)
+    int32_t part;
+};
+struct MarchArgs {
+    FusedArgs f;              // buffers, hyp, ctl, key, update (its tiles are unused)
+    const MarchTile *tiles;
+    int32_t ntiles;
+    int32_t intercept;        // the model has the intercept (its sum is then compensated)
+    uint32_t rk[20];          // Philox round keys
+    // the batch form only
+    HyperArgs h;
+    int32_t count;
+    int32_t zrows;            // rows of a chunk whose normals are drawn ahead
+    double *pm;               // [Cp][S, R, A][block]
+    uint32_t extra_arrivals;
+    uint64_t wait_ns;
+};
+int march_warps();            // chunks of a block
+int march_strips(int kind, int Cp, int W);
+int march_blocks(int kind, int Cp, int H, int W, int rows);
+int march_ahead_rows(int Cp, int rows);
+cudaError_t plan_march_grid(int kind, int Cp, int blocks, int zrows, bool *fits);
+cudaError_t launch_march(int kind, const MarchArgs &a, cudaStream_t stream);
+cudaError_t launch_march_grid(int kind, const MarchArgs &a, cudaStream_t stream);
+
 // Jones-Plassmann colouring and colour-permuted CSR layout (csr_build.cu).
 struct CsrBuild {
     int32_t n;

@@ -147,31 +147,28 @@ __device__ __forceinline__ void hyper_sums(const HyperArgs &a, int which, bool n
     const int lane = threadIdx.x & 31;
     const Part3 *P = a.partials + static_cast<int64_t>(part0) * a.Cp + chain;
     if constexpr (BATCH) {
-        double rs[kSumRows], ra[kSumRows];
+        double vs[kSumRows], va[kSumRows];  // the lane's rows
 #pragma unroll
         for (int j = 0; j < kSumRows; ++j) {
-            rs[j] = 0.0;
-            ra[j] = 0.0;
+            const int k = lane + 32 * j;
+            vs[j] = 0.0;
+            va[j] = 0.0;
+            if (k < nparts) part_values<CG>(P + static_cast<int64_t>(k) * a.Cp, which, need_a, vs[j], va[j]);
         }
-        for (int k0 = lane; k0 < nparts; k0 += 32 * kSumRows) {
-            double vs[kSumRows], va[kSumRows];
+        for (int k0 = lane + 32 * kSumRows; k0 < nparts; k0 += 32 * kSumRows) {
 #pragma unroll
             for (int j = 0; j < kSumRows; ++j) {
-                vs[j] = 0.0;
-                va[j] = 0.0;
-                if (k0 + 32 * j < nparts)
-                    part_values<CG>(P + static_cast<int64_t>(k0 + 32 * j) * a.Cp, which, need_a, vs[j], va[j]);
-            }
-#pragma unroll
-            for (int j = 0; j < kSumRows; ++j) {
-                rs[j] += vs[j];
-                if (need_a) ra[j] += va[j];
+                if (k0 + 32 * j >= nparts) continue;
+                double v, w;
+                part_values<CG>(P + static_cast<int64_t>(k0 + 32 * j) * a.Cp, which, need_a, v, w);
+                vs[j] += v;
+                if (need_a) va[j] += w;
             }
         }
 #pragma unroll
         for (int j = 0; j < kSumRows; ++j) {
-            S += rs[j];
-            if (need_a) A += ra[j];
+            S += vs[j];
+            if (need_a) A += va[j];
         }
     } else {  // at most 256 partials
         for (int k = lane; k < nparts; k += 32) {
