@@ -1505,13 +1505,18 @@ gmrf_status build_chromatic(gmrf_sampler *s, const gmrf_field_desc *fields, std:
             // worth 1024 site updates (fitted to measured 20 x 22 and 64 x 64 tilings of many
             // small lattices).  Deterministic, so a sampler's tiling (and with it the rounding of
             // the tile partial sums) does not change from run to run.
+            // (FP64, whose site updates cost some thirty times as much: a block's fixed cost is worth 200,
+            // and 4-neighbour tiles go down to 8 x 8: 64 x 64 sites, one chain 13.0 -> 11.2 us per sweep,
+            // 128 x 129, four chains 52 -> 34; the 8-neighbour halo of four leaves 100 x 131 2 % slower)
+            const double block_cost = s->precision == GMRF_FP32 ? 1024.0 : 200.0;
+            const int least_side = s->precision == GMRF_FP64 && K == 2 ? 8 : 16;
             double best = 1e300;
             for (int nt : {512, 1024}) {
                 // blocks per SM: two of 512 threads where the kernel is compiled for 64 registers
                 // (FP32 with up to two chains per thread), else one (four chains keep 128)
                 const int bps = (nt == 512 && s->precision == GMRF_FP32 && s->Cp < 4) ? 2 : 1;
-                for (int cr = 16; cr <= 160; cr += 2)
-                    for (int cc = 16; cc <= 128; cc += 2) {
+                for (int cr = least_side; cr <= 160; cr += 2)
+                    for (int cc = least_side; cc <= 128; cc += 2) {
                         const size_t sm = lattice_fused_smem(s->precision, kind, s->Cp, cr, cc);
                         if (sm * bps > 200 * 1024 || static_cast<int64_t>(cr + 2 * K) * (cc + 2 * K) * s->Cp >= 65536)
                             continue;
@@ -1519,7 +1524,7 @@ gmrf_status build_chromatic(gmrf_sampler *s, const gmrf_field_desc *fields, std:
                         for (auto &h : s->hf)
                             if (h.kind == kind)
                                 tiles += static_cast<int64_t>((h.dims[0] + cr - 1) / cr) * ((h.dims[1] + cc - 1) / cc);
-                        double work = 1024.0;  // per block: fixed cost + sites computed over the K steps
+                        double work = block_cost;  // per block: fixed cost + sites computed over the K steps
                         for (int e = 0; e < K; ++e) work += static_cast<double>(cr + 2 * e) * (cc + 2 * e) / K;
                         const double waves = std::ceil(static_cast<double>(tiles) / (152.0 * bps));
                         const double cost = waves * bps * work;
@@ -1556,8 +1561,13 @@ gmrf_status build_chromatic(gmrf_sampler *s, const gmrf_field_desc *fields, std:
     for (int fi = 0; fi < s->nfields; ++fi)
         if (!fused_kind[s->hf[fi].kind]) total_elems += static_cast<int64_t>(s->hf[fi].n) * CV;
     const int64_t per_colour = total_elems / 2;
+    // (FP64: a step is bound by the SMs' FP64 pipes, so a class of fewer elements than the SMs have
+    // threads is spread over all of them, down to 64 elements per tile: 30 x 30 x 31 sites, one chain,
+    // 42 -> 32 us per sweep; but no smaller tiles than one per SM, 48^3 with two chains 80 -> 142)
+    const int64_t least = s->precision == GMRF_FP32 ? kBlock
+                                                    : std::min<int64_t>(kBlock, std::max<int64_t>(64, per_colour / 140));
     const int64_t target = s->tune.step_tile ? s->tune.step_tile
-                                             : std::min<int64_t>(16384, std::max<int64_t>(kBlock, per_colour / (152 * 4)));
+                                             : std::min<int64_t>(16384, std::max<int64_t>(least, per_colour / (152 * 4)));
     // 3-D lattices with every chain of a site in one thread: FP32, 4 or 8 chains (padded), the
     // Gaussian likelihood, and either asked for (tuning.wide_3d = 1) or, by default, colour
     // classes of at least one site for each of 256 threads on every SM.  A launch is then one
@@ -1931,7 +1941,8 @@ gmrf_status gmrf_sampler_create(gmrf_sampler **out, const gmrf_field_desc *field
         // Samplers whose sweeps are per-colour launches only (3-D lattices, graphs): when a step
         // has too few (site, chain group) elements to fill the GPU (below 2048 threads on each of
         // the 152 SMs, four times over), fewer chains per thread give more threads.  (Fused 2-D
-        // sweeps keep all chains in a thread: their fast kernel needs it.)
+        // sweeps keep all chains in a thread: their fast kernel needs it.  FP64 keeps two: a step
+        // is bound by the FP64 pipe, and a Box-Muller pair then serves a thread's two chains.)
         bool lattice2d = false;
         int64_t sites = 0;
         for (const HostField &h : hf) {
@@ -1939,7 +1950,7 @@ gmrf_status gmrf_sampler_create(gmrf_sampler **out, const gmrf_field_desc *field
                          !(opts->flags & GMRF_FLAG_PER_COLOUR);
             sites += h.n;
         }
-        while (!lattice2d && s->V > 1 && sites * s->Cp / s->V < int64_t(152) * 2048 * 4) s->V >>= 1;
+        while (!lattice2d && s->V > (opts->precision == GMRF_FP64 ? 2 : 1) && sites * s->Cp / s->V < int64_t(152) * 2048 * 4) s->V >>= 1;
     }
     if (s->tune.chains_per_thread) s->V = s->tune.chains_per_thread;
     s->algorithm = opts->algorithm;

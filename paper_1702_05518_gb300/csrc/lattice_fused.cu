@@ -25,6 +25,20 @@
 namespace gmrf {
 namespace {
 
+// FP64: 1/P and 1/sqrt(P) per degree and chain ([degree][Cp][2], shared memory).  P takes no other
+// values on a lattice, and two FP64 quotients and a root per site were a third of its FP64 operations.
+template <typename T> constexpr bool kDegreeTable = sizeof(T) == 8;
+template <typename T>
+__device__ __forceinline__ void degree_table(T *tab, const T *hyp, int Cp, int threads)
+{
+    if constexpr (kDegreeTable<T>)
+        for (int q = threadIdx.x; q < 9 * Cp; q += threads) {
+            const int dg = q / Cp, v = q - dg * Cp;
+            const T P = hyp[v * kHypStride] * static_cast<T>(dg) + hyp[v * kHypStride + 1];
+            tab[2 * q] = FArith<T>::rcp(P);
+            tab[2 * q + 1] = FArith<T>::rsq(P);
+        }
+}
 template <typename T, int V, int KIND, int kFusedBlock>
 __global__ void __launch_bounds__(kFusedBlock, (kFusedBlock == 512 && sizeof(T) == 4 && V <= 2) ? 2 : 1)
     lattice_fused_kernel(const FusedArgs a)
@@ -61,6 +75,7 @@ __global__ void __launch_bounds__(kFusedBlock, (kFusedBlock == 512 && sizeof(T) 
     const uint32_t sweep = static_cast<uint32_t>(sweep_ll);
     const T rho = static_cast<T>(a.rho);
 
+    __shared__ T tab[kDegreeTable<T> ? 9 * kMaxChains * 2 : 1];
     T tau[V], isig[V], beta[V];
     const T *hyp = static_cast<const T *>(a.hyp);
 #pragma unroll
@@ -70,6 +85,8 @@ __global__ void __launch_bounds__(kFusedBlock, (kFusedBlock == 512 && sizeof(T) 
         isig[v] = hyp[hc + 1];
         beta[v] = hyp[hc + 2];
     }
+
+    degree_table(tab, hyp + static_cast<int64_t>(t.field) * Cp * kHypStride, Cp, kFusedBlock);
 
     // Stage: rows of the NS sub-arrays; slots outside a global sub-array read as zero, and the
     // global padding slots (sites beyond an odd extent) hold zero, so every position outside
@@ -260,9 +277,15 @@ __global__ void __launch_bounds__(kFusedBlock, (kFusedBlock == 512 && sizeof(T) 
             T xn[V];
 #pragma unroll
             for (int v = 0; v < V; ++v) {
-                const T P = tau[v] * d + isig[v];
-                const T m = (tau[v] * rho * s[v] + (yv - beta[v]) * isig[v]) * FArith<T>::rcp(P);
-                xn[v] = m + z[v] * FArith<T>::rsq(P);
+                if constexpr (kDegreeTable<T>) {
+                    const T *q = tab + (deg * Cp + cvo + v) * 2;
+                    const T m = (tau[v] * rho * s[v] + (yv - beta[v]) * isig[v]) * q[0];
+                    xn[v] = m + z[v] * q[1];
+                } else {
+                    const T P = tau[v] * d + isig[v];
+                    const T m = (tau[v] * rho * s[v] + (yv - beta[v]) * isig[v]) * FArith<T>::rcp(P);
+                    xn[v] = m + z[v] * FArith<T>::rsq(P);
+                }
             }
             Vec<T, V>::st(xs + idx * Cp + cvo, xn);
             if (i >= t.i0 && i < t.i0 + TR && j >= t.j0 && j < t.j0 + TC) {
@@ -545,6 +568,8 @@ __global__ void __launch_bounds__(NT, (NT == 512 && sizeof(T) == 4 && CP < 4) ? 
             beta[v] = hyp[kHypStride * v + 2];
         }
     }
+    __shared__ T tab[kDegreeTable<T> ? 9 * CP * 2 : 1];
+    degree_table(tab, static_cast<const T *>(a.hyp) + static_cast<int64_t>(t.field) * CP * kHypStride, CP, NT);
     stage(X, nullptr);
     __syncthreads();
 
@@ -646,6 +671,7 @@ __global__ void __launch_bounds__(NT, (NT == 512 && sizeof(T) == 4 && CP < 4) ? 
                     for (int v = 0; v < CP; ++v) s[v] += nb[k][v];
                 }
                 T d = static_cast<T>(ND);
+                int dg = ND;
                 T wv[ND];
 #pragma unroll
                 for (int k = 0; k < ND; ++k) wv[k] = wl[k];
@@ -661,6 +687,7 @@ __global__ void __launch_bounds__(NT, (NT == 512 && sizeof(T) == 4 && CP < 4) ? 
                         if (!ok) wv[k] = 0;
                     }
                     d = static_cast<T>(deg);
+                    dg = deg;
                 }
                 T z[CP];
                 Vec<T, CP>::ld(zs + idx * CP, z);
@@ -668,9 +695,15 @@ __global__ void __launch_bounds__(NT, (NT == 512 && sizeof(T) == 4 && CP < 4) ? 
                 T xn[CP];
 #pragma unroll
                 for (int v = 0; v < CP; ++v) {
-                    const T P = tau[v] * d + isig[v];
-                    const T m = (tau[v] * rho * s[v] + (yv - beta[v]) * isig[v]) * FArith<T>::rcp(P);
-                    xn[v] = m + z[v] * FArith<T>::rsq(P);
+                    if constexpr (kDegreeTable<T>) {
+                        const T *q = tab + (dg * CP + v) * 2;
+                        const T m = (tau[v] * rho * s[v] + (yv - beta[v]) * isig[v]) * q[0];
+                        xn[v] = m + z[v] * q[1];
+                    } else {
+                        const T P = tau[v] * d + isig[v];
+                        const T m = (tau[v] * rho * s[v] + (yv - beta[v]) * isig[v]) * FArith<T>::rcp(P);
+                        xn[v] = m + z[v] * FArith<T>::rsq(P);
+                    }
                 }
                 Vec<T, CP>::st(xs + idx * CP, xn);
                 if (owned) {

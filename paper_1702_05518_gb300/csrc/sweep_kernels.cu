@@ -53,7 +53,13 @@ struct SiteCtx {
     T accS[V], accR[V], accA[V]; // thread partial sums
     T inv_k;             // 1 / (accumulated count) when accumulating
     bool acc;
+    // FP64 lattices: 1/P and 1/sqrt(P) per degree and chain ([degree][Cp][2], shared memory).  P takes
+    // no other values without weights, and the two FP64 quotients and the root were a third of a site's
+    // FP64 operations.
+    const T *tab;
 };
+// Whether a kernel uses that table.
+template <typename T, int KIND, int MODEL> constexpr bool kDegreeTable = sizeof(T) == 8 && KIND != kCsr && MODEL != kModelBinomial;
 
 // Draw (or, in reduce-only mode, read) the V chain values of one site given its neighbour sum s
 // and the neighbour values nb[k] of the neighbours flagged in `lower_mask` (those of lower
@@ -64,7 +70,7 @@ struct SiteCtx {
 // (tau rho s_i + kappa_i - psi beta0) / P,
 // kappa_i = y_i - m_i / 2; the partial sums then collect psi and kappa_i - psi x_i (for beta0)
 // in place of the Gaussian residual sums.
-template <typename T, int V, int NB, int MODEL>
+template <typename T, int V, int NB, int MODEL, bool TAB = false>
 __device__ __forceinline__ void finish_site(const StepArgs &a, SiteCtx<T, V> &cx, T *xp, T *meanp, T *m2p,
                                             T yv, int mtr, T d, uint32_t site, uint32_t sweep, uint32_t stream,
                                             uint32_t chain0, const T (&s)[V], const T (&nb)[NB][V],
@@ -99,9 +105,15 @@ __device__ __forceinline__ void finish_site(const StepArgs &a, SiteCtx<T, V> &cx
         site_normals<T, V>(a.key, site, sweep, stream, chain0, a.lanes, z);
 #pragma unroll
         for (int v = 0; v < V; ++v) {
-            const T P = cx.tau[v] * d + cx.isig[v];
-            const T m = (cx.tau[v] * rho * s[v] + (yv - cx.beta[v]) * cx.isig[v]) * Arith<T>::rcp(P);
-            xn[v] = m + z[v] * Arith<T>::rsq(P);
+            if constexpr (TAB) {
+                const T *q = cx.tab + (static_cast<int>(d) * a.Cp + static_cast<int>(chain0) + v) * 2;
+                const T m = (cx.tau[v] * rho * s[v] + (yv - cx.beta[v]) * cx.isig[v]) * q[0];
+                xn[v] = m + z[v] * q[1];
+            } else {
+                const T P = cx.tau[v] * d + cx.isig[v];
+                const T m = (cx.tau[v] * rho * s[v] + (yv - cx.beta[v]) * cx.isig[v]) * Arith<T>::rcp(P);
+                xn[v] = m + z[v] * Arith<T>::rsq(P);
+            }
         }
         Vec<T, V>::st(xp, xn);
     } else {
@@ -217,7 +229,7 @@ __device__ void lattice_parity_tile(const StepArgs &a, const FieldDev &f, const 
         }
         const uint32_t site = static_cast<uint32_t>(r * W + j);
         const int mtr = MODEL == kModelBinomial ? a.trials[self_base + rb] : 0;
-        finish_site<T, V, NB, MODEL>(a, cx, XS + rb * Cp, MS + rb * Cp, QS + rb * Cp, YS[rb], mtr, static_cast<T>(__popc(valid)),
+        finish_site<T, V, NB, MODEL, kDegreeTable<T, kLat3D6, MODEL>>(a, cx, XS + rb * Cp, MS + rb * Cp, QS + rb * Cp, YS[rb], mtr, static_cast<T>(__popc(valid)),
                               site, sweep, f.stream, static_cast<uint32_t>(cv * V), s, nb, lower_all & valid, wnb);
     }
 }
@@ -296,7 +308,7 @@ __device__ void lattice8_tile(const StepArgs &a, const FieldDev &f, const Tile &
         }
         const uint32_t site = static_cast<uint32_t>(i * W + j);
         const int mtr = MODEL == kModelBinomial ? a.trials[f.slot0 + static_cast<int64_t>(c) * sub + base] : 0;
-        finish_site<T, V, NB, MODEL>(a, cx, XS + base * Cp, MS + base * Cp, QS + base * Cp, YS[base], mtr,
+        finish_site<T, V, NB, MODEL, kDegreeTable<T, kLat2D8, MODEL>>(a, cx, XS + base * Cp, MS + base * Cp, QS + base * Cp, YS[base], mtr,
                               static_cast<T>(__popc(valid)), site, sweep, f.stream, static_cast<uint32_t>(cv * V),
                               s, nb, lower & valid, wnb);
     }
@@ -417,6 +429,19 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? (KIND == kCsr ? 2 : 3
     if (a.update && a.acc_enabled && sweep_accumulated(sweep_ll, a.burn_in, a.thin)) {
         cx.acc = true;
         cx.inv_k = static_cast<T>(1) / static_cast<T>(a.ctl->acc_count + 1);
+    }
+
+    __shared__ T tab[kDegreeTable<T, KIND, MODEL> ? 9 * kMaxChains * 2 : 1];
+    cx.tab = tab;
+    if constexpr (kDegreeTable<T, KIND, MODEL>) {
+        for (int q = threadIdx.x; q < 9 * a.Cp; q += kBlock) {
+            const int dg = q / a.Cp, v = q - dg * a.Cp;
+            const T *hv = hyp + (static_cast<int64_t>(t.field) * a.Cp + v) * kHypStride;
+            const T P = hv[0] * static_cast<T>(dg) + hv[1];
+            tab[2 * q] = Arith<T>::rcp(P);
+            tab[2 * q + 1] = Arith<T>::rsq(P);
+        }
+        __syncthreads();
     }
 
     const int cv_shift = __ffs(CV) - 1;
