@@ -568,70 +568,127 @@ __global__ void __launch_bounds__(kSumRows * 32) hyper_wide_kernel(const HyperAr
     hyper_end(a, sweep);
 }
 
-// The Polya-Gamma stage of the binomial model: one warp per (slot, chain).  The slot's natural
-// site gives the counters; lane l draws the PG(1, c) summands k = l, l + 32, ... < m_i and the
-// warp adds them in a fixed order (shuffle tree); psi = 0 for sites without trials and for
-// padding slots.
-template <typename T>
-__global__ void pg_stage_kernel(const PgArgs a)
+// The Polya-Gamma stage of the binomial model: psi of (slot, chain) is the sum of m_i draws of
+// PG(1, c); psi = 0 for sites without trials and for padding slots.  A block takes kPgSlots (slot,
+// chain) pairs and spreads their draws over its threads in one sequence, so that a warp's lanes are
+// full whatever the m_i (with a warp per pair half the lanes had no draw, and the proposal's mixture
+// weight, a dozen special functions, was computed by one lane of each warp; here by one thread per
+// pair).  A pair's draws are added in a fixed order that does not depend on the block: draw k into
+// lane k mod 32 in turn, then a shuffle tree over the lanes.  Bound by the instructions of the
+// rejection loops and their divergence (16 of 32 lanes active, 49 % issue): 14,926 sites with 226,000
+// draws 34 -> 22 us.
+constexpr int kPgSlots = 32, kPgThreads = 256, kPgPass = 1024;  // kPgPass: draws between barriers
+
+// Natural site of a slot of field f (rel: relative to the field), -1 for the padding of a lattice layout.
+__device__ __forceinline__ int64_t site_of_slot(const PgArgs &a, const FieldDev &f, int64_t rel)
 {
+    if (f.kind == kCsr) return a.perm[f.csr0 + rel];
+    const int64_t sub = static_cast<int64_t>(f.rows) * f.cols;
+    const int64_t c = rel / sub, r = (rel - c * sub) / f.cols, h = rel - c * sub - r * f.cols;
+    if (f.kind == kLat2D8) {
+        const int64_t i = 2 * r + (c >> 1), j = 2 * h + (c & 1);
+        return (i < f.dims[0] && j < f.dims[1]) ? i * f.dims[1] + j : -1;
+    }
+    if (f.kind == kLat2D4) {
+        const int64_t j = 2 * h + ((c + r) & 1);
+        return j < f.dims[1] ? r * f.dims[1] + j : -1;
+    }
+    const int64_t l = r / f.dims[1], i = r - l * f.dims[1], j = 2 * h + ((c + l + i) & 1);
+    return j < f.dims[2] ? r * f.dims[2] + j : -1;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kPgThreads) pg_stage_kernel(const PgArgs a)
+{
+    __shared__ T s_z[kPgSlots], s_w[kPgSlots], s_val[kPgPass], s_acc[kPgSlots][32];
+    __shared__ int s_end[kPgSlots];  // draws of the block's pairs up to and with this one
+    __shared__ uint32_t s_site[kPgSlots], s_chain[kPgSlots], s_stream[kPgSlots];
     pdl_wait_then_release();
-    const int lane = threadIdx.x & 31;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t sweep = static_cast<uint32_t>(a.ctl->sweep);
-    const int64_t warps = static_cast<int64_t>(gridDim.x) * (blockDim.x >> 5);
     const T *X = static_cast<const T *>(a.x);
     const T *hyp = static_cast<const T *>(a.hyp);
     T *PSI = static_cast<T *>(a.psi);
+    const int64_t tasks = a.slots * a.C;
     int fb = 0;
-    for (int64_t task = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; task < a.slots * a.C;
-         task += warps) {
-        const int64_t slot = task / a.C;
-        const int chain = static_cast<int>(task - slot * a.C);
-        int fi = 0;  // field of the slot (fields are few; their slot ranges are in order)
-        while (fi + 1 < a.nfields && a.fields[fi + 1].slot0 <= slot) ++fi;
-        const FieldDev &f = a.fields[fi];
-        const int64_t rel = slot - f.slot0;
-        // natural site of the slot (padding slots of the lattice layouts have none)
-        int64_t site = -1;
-        if (f.kind == kCsr) {
-            site = a.perm[f.csr0 + rel];
-        } else {
-            const int64_t sub = static_cast<int64_t>(f.rows) * f.cols;
-            const int64_t c = rel / sub, r = (rel - c * sub) / f.cols, h = rel - c * sub - r * f.cols;
-            if (f.kind == kLat2D8) {
-                const int64_t i = 2 * r + (c >> 1), j = 2 * h + (c & 1);
-                if (i < f.dims[0] && j < f.dims[1]) site = i * f.dims[1] + j;
-            } else if (f.kind == kLat2D4) {
-                const int64_t j = 2 * h + ((c + r) & 1);
-                if (j < f.dims[1]) site = r * f.dims[1] + j;
-            } else {
-                const int64_t l = r / f.dims[1], i = r - l * f.dims[1], j = 2 * h + ((c + l + i) & 1);
-                if (j < f.dims[2]) site = r * f.dims[2] + j;
+    for (int64_t first = static_cast<int64_t>(blockIdx.x) * kPgSlots; first < tasks;
+         first += static_cast<int64_t>(gridDim.x) * kPgSlots) {
+        for (int q = tid; q < kPgSlots * 32; q += kPgThreads) s_acc[q >> 5][q & 31] = 0;
+        if (warp == 0) {
+            static_assert(kPgSlots == 32, "a pair per lane of the first warp");
+            const int64_t task = first + lane;
+            int m = 0;
+            if (task < tasks) {
+                const int64_t slot = task / a.C;
+                const int chain = static_cast<int>(task - slot * a.C);
+                int fi = 0;  // field of the slot (fields are few; their slot ranges are in order)
+                while (fi + 1 < a.nfields && a.fields[fi + 1].slot0 <= slot) ++fi;
+                const FieldDev &f = a.fields[fi];
+                const int64_t site = site_of_slot(a, f, slot - f.slot0);
+                m = site >= 0 ? a.trials[slot] : 0;
+                if (m > 0) {
+                    const T eta = hyp[(static_cast<int64_t>(fi) * a.Cp + chain) * kHypStride + 2] + X[slot * a.Cp + chain];
+                    // the sampler's arithmetic follows the state precision (pg.cuh)
+                    const T z = static_cast<T>(0.5) * fabs(eta);
+                    s_z[lane] = z;
+                    s_w[lane] = pg_exp_weight<T>(z);
+                    s_site[lane] = static_cast<uint32_t>(site);
+                    s_chain[lane] = static_cast<uint32_t>(chain);
+                    s_stream[lane] = f.stream;
+                }
             }
+            int end = m;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, end, o);
+                if (lane >= o) end += v;
+            }
+            s_end[lane] = end;
         }
-        const int m = site >= 0 ? a.trials[slot] : 0;
-        // the sampler's arithmetic follows the state precision (pg.cuh)
-        T sum = 0;
-        if (m > 0) {
-            const T eta = hyp[(static_cast<int64_t>(fi) * a.Cp + chain) * kHypStride + 2] + X[slot * a.Cp + chain];
-            const T z = static_cast<T>(0.5) * fabs(eta);
-            // the proposal's mixture weight, once per warp (the special functions are costly)
-            T wexp = lane == 0 ? pg_exp_weight<T>(z) : static_cast<T>(0);
-            wexp = __shfl_sync(0xffffffffu, wexp, 0);
-            for (int k = lane; k < m; k += 32) {
+        __syncthreads();
+        const int total = s_end[kPgSlots - 1];
+        auto pair_of = [&](int q) {  // the first pair that ends beyond draw q
+            int p = 0;
+#pragma unroll
+            for (int o = kPgSlots / 2; o >= 1; o >>= 1)
+                if (s_end[p + o - 1] <= q) p += o;
+            return p;
+        };
+        for (int q0 = 0; q0 < total; q0 += kPgPass) {
+            const int q1 = min(total, q0 + kPgPass);
+            for (int q = q0 + tid; q < q1; q += kPgThreads) {
+                const int p = pair_of(q), start = p > 0 ? s_end[p - 1] : 0;
                 PgStream st;
-                pg_stream_init(st, a.key, static_cast<uint32_t>(site), sweep, f.stream, static_cast<uint32_t>(chain),
-                               static_cast<uint32_t>(k));
-                T j = pg_jstar<T>(z, wexp, st);
+                pg_stream_init(st, a.key, s_site[p], sweep, s_stream[p], s_chain[p], static_cast<uint32_t>(q - start));
+                const T z = s_z[p];
+                T j = pg_jstar<T>(z, s_w[p], st);
                 if (j < static_cast<T>(0)) {
                     ++fb;
                     j = z > static_cast<T>(0) ? tanh(z) / z : static_cast<T>(1);
                 }
-                sum += static_cast<T>(0.25) * j;
+                s_val[q - q0] = static_cast<T>(0.25) * j;
+            }
+            __syncthreads();
+            // the pass's draws into the pairs' lanes, by the thread of a lane's first draw in the pass
+            for (int q = q0 + tid; q < q1; q += kPgThreads) {
+                const int p = pair_of(q), start = p > 0 ? s_end[p - 1] : 0;
+                if (q - max(start, q0) >= 32) continue;
+                const int end = min(s_end[p], q1);
+                T acc = s_acc[p][(q - start) & 31];
+                for (int k = q; k < end; k += 32) acc += s_val[k - q0];
+                s_acc[p][(q - start) & 31] = acc;
+            }
+            __syncthreads();
+        }
+        for (int p = warp; p < kPgSlots; p += kPgThreads / 32) {
+            T sum = s_acc[p][lane];
+            for (int off = 16; off >= 1; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+            if (lane == 0 && first + p < tasks) {
+                const int64_t slot = (first + p) / a.C;
+                PSI[slot * a.Cp + (first + p - slot * a.C)] = sum;
             }
         }
-        for (int off = 16; off >= 1; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
-        if (lane == 0) PSI[slot * a.Cp + chain] = sum;
+        __syncthreads();
     }
     if (fb) atomicAdd(reinterpret_cast<unsigned long long *>(&a.ctl->fallbacks), static_cast<unsigned long long>(fb));
 }
@@ -871,11 +928,11 @@ cudaError_t launch_pack(int precision, const FieldDev *fields_dev, const FieldDe
 cudaError_t launch_pg_stage(int precision, const PgArgs &a, cudaStream_t stream)
 {
     const int64_t tasks = a.slots * a.C;
-    int64_t blocks = (tasks + 7) / 8;  // eight warps per block
+    int64_t blocks = (tasks + kPgSlots - 1) / kPgSlots;
     if (blocks > 152 * 64) blocks = 152 * 64;
     if (blocks < 1) blocks = 1;
-    if (precision == 0) return launch_sweep_kernel(pg_stage_kernel<float>, static_cast<int>(blocks), 256, 0, stream, a);
-    return launch_sweep_kernel(pg_stage_kernel<double>, static_cast<int>(blocks), 256, 0, stream, a);
+    if (precision == 0) return launch_sweep_kernel(pg_stage_kernel<float>, static_cast<int>(blocks), kPgThreads, 0, stream, a);
+    return launch_sweep_kernel(pg_stage_kernel<double>, static_cast<int>(blocks), kPgThreads, 0, stream, a);
 }
 
 namespace {
