@@ -63,7 +63,7 @@ template <typename T, int KIND, int MODEL> constexpr bool kDegreeTable = sizeof(
 
 // Draw (or, in reduce-only mode, read) the V chain values of one site given its neighbour sum s
 // and the neighbour values nb[k] of the neighbours flagged in `lower_mask` (those of lower
-// colour), and fold the site's terms into the partial sums.
+// colour), and fold the site's terms into the partial sums.  zdrawn: its normals if already drawn.
 //
 // Binomial model: psi | beta0, x_i ~ PG(m_i, beta0 + x_i) was drawn from the site's value at the
 // start of the sweep (the Polya-Gamma stage); x_i gets precision tau d_i + psi and mean
@@ -74,7 +74,7 @@ template <typename T, int V, int NB, int MODEL, bool TAB = false>
 __device__ __forceinline__ void finish_site(const StepArgs &a, SiteCtx<T, V> &cx, T *xp, T *meanp, T *m2p,
                                             T yv, int mtr, T d, uint32_t site, uint32_t sweep, uint32_t stream,
                                             uint32_t chain0, const T (&s)[V], const T (&nb)[NB][V],
-                                            uint32_t lower_mask, const T (&wnb)[NB])
+                                            uint32_t lower_mask, const T (&wnb)[NB], const T *zdrawn = nullptr)
 {
     const T rho = static_cast<T>(a.rho);
     T xn[V];
@@ -92,7 +92,12 @@ __device__ __forceinline__ void finish_site(const StepArgs &a, SiteCtx<T, V> &cx
         T z[V];
         // psi of this site and chain, drawn by the Polya-Gamma stage from the start-of-sweep state
         Vec<T, V>::ld(static_cast<const T *>(a.psi) + (xp - static_cast<T *>(a.x)), psi);
-        site_normals<T, V>(a.key, site, sweep, stream, chain0, a.lanes, z);
+        if (zdrawn) {
+#pragma unroll
+            for (int v = 0; v < V; ++v) z[v] = zdrawn[v];
+        } else {
+            site_normals<T, V>(a.key, site, sweep, stream, chain0, a.lanes, z);
+        }
 #pragma unroll
         for (int v = 0; v < V; ++v) {
             const T P = cx.tau[v] * d + psi[v];
@@ -102,7 +107,12 @@ __device__ __forceinline__ void finish_site(const StepArgs &a, SiteCtx<T, V> &cx
         Vec<T, V>::st(xp, xn);
     } else if (a.update) {
         T z[V];
-        site_normals<T, V>(a.key, site, sweep, stream, chain0, a.lanes, z);
+        if (zdrawn) {
+#pragma unroll
+            for (int v = 0; v < V; ++v) z[v] = zdrawn[v];
+        } else {
+            site_normals<T, V>(a.key, site, sweep, stream, chain0, a.lanes, z);
+        }
 #pragma unroll
         for (int v = 0; v < V; ++v) {
             if constexpr (TAB) {
@@ -314,52 +324,97 @@ __device__ void lattice8_tile(const StepArgs &a, const FieldDev &f, const Tile &
     }
 }
 
+// The neighbours of a row that stay in registers: their loads are all issued before any is used, and the
+// lower-colour terms of the prior sum need no second pass over them.
+template <int V> constexpr int kCsrRow = V == 4 ? 6 : 8;
+
+// One position of a CSR field: what no kernel of a sweep writes (row, weights, degree, observation,
+// site), and its normals when drawn.  A block loads its threads' first positions before it waits for the
+// previous colour step (csr_ahead), so that after the wait only the neighbours' values are left to gather.
+template <typename T, int V>
+struct CsrSite {
+    int pos, rb, re, jn[kCsrRow<V>], mtr;
+    T wnb[kCsrRow<V>], yv, d, z[V];
+    uint32_t site, sweep;  // sweep: of the normals
+    bool drawn;
+};
+
+template <typename T, int V, int MODEL>
+__device__ __forceinline__ void csr_load(const StepArgs &a, const FieldDev &f, int pos, CsrSite<T, V> &c)
+{
+    const int32_t *rp = a.rp + f.rp0, *ci = a.ci + f.nnz0;
+    const T *wr = a.w ? static_cast<const T *>(a.w) + f.nnz0 : nullptr;
+    c.pos = pos;
+    c.rb = rp[pos];
+    c.re = rp[pos + 1];
+#pragma unroll
+    for (int q = 0; q < kCsrRow<V>; ++q) {
+        const int k = c.rb + q;
+        c.jn[q] = k < c.re ? ci[k] : -1;
+        c.wnb[q] = k < c.re ? (wr ? wr[k] : static_cast<T>(1)) : static_cast<T>(0);
+    }
+    c.yv = static_cast<const T *>(a.y)[f.slot0 + pos];
+    c.d = static_cast<const T *>(a.deg)[f.csr0 + pos];
+    c.site = static_cast<uint32_t>(a.perm[f.csr0 + pos]);
+    c.mtr = MODEL == kModelBinomial ? a.trials[f.slot0 + pos] : 0;
+    c.drawn = false;
+}
+
+// The thread's first position, before the dependency wait (pos < 0: none).  From colour 1 on the
+// normals too: the previous launch is a colour step of the same sweep, which let this one start after
+// its own wait, so everything before it, the draws that advanced the sweep number included, is complete
+// (csr_tile checks the number all the same: a stage launched alone may follow another kernel).
+template <typename T, int V, int MODEL>
+__device__ __forceinline__ void csr_ahead(const StepArgs &a, const FieldDev &f, const Tile &t, CsrSite<T, V> &c)
+{
+    const int CV = a.Cp / V, e = threadIdx.x;
+    c.pos = -1;
+    if (e >= t.count * CV) return;
+    csr_load<T, V, MODEL>(a, f, t.start + e / CV, c);
+    if (a.update && t.colour > 0) {
+        c.sweep = static_cast<uint32_t>(*reinterpret_cast<volatile const long long *>(&a.ctl->sweep));
+        site_normals<T, V>(a.key, c.site, c.sweep, f.stream, static_cast<uint32_t>((e % CV) * V), a.lanes, c.z);
+        c.drawn = true;
+    }
+}
+
 // CSR field: permuted positions [start, start + count) of one colour class; neighbours are read
 // through the permuted row; a neighbour has lower colour iff its position is below the class's
 // first position.
 template <typename T, int V, int MODEL>
 __device__ void csr_tile(const StepArgs &a, const FieldDev &f, const Tile &t, SiteCtx<T, V> &cx, int CV,
-                         int cv_shift, uint32_t sweep)
+                         int cv_shift, uint32_t sweep, CsrSite<T, V> &c)
 {
     T *X = static_cast<T *>(a.x);
-    const T *Y = static_cast<const T *>(a.y);
     T *MEAN = static_cast<T *>(a.mean);
     T *M2 = static_cast<T *>(a.m2);
     const T *Wt = static_cast<const T *>(a.w);
-    const T *DEG = static_cast<const T *>(a.deg);
     const int64_t Cp = a.Cp;
-    const int32_t *rp = a.rp + f.rp0;
     const int32_t *ci = a.ci + f.nnz0;
     const T *wr = Wt ? Wt + f.nnz0 : nullptr;
     const int32_t lo = a.coff[f.coff0 + t.colour];
     const T rho = static_cast<T>(a.rho);
     const int nelem = t.count * CV;
+    constexpr int R = kCsrRow<V>;
     for (int e = threadIdx.x; e < nelem; e += kBlock) {
         const int cv = e & (CV - 1);
-        const int pos = t.start + (e >> cv_shift);
-        const int rb = rp[pos], re = rp[pos + 1];
-        // The first R neighbours stay in registers: their loads are all issued before any is
-        // used, and the lower-colour terms of the prior sum need no second pass over them.
-        constexpr int R = V == 4 ? 6 : 8;
-        T nb[R][V], wnb[R], s[V];
+        if (e != static_cast<int>(threadIdx.x)) csr_load<T, V, MODEL>(a, f, t.start + (e >> cv_shift), c);
+        const int pos = c.pos, rb = c.rb, re = c.re;
+        T nb[R][V], s[V];
         uint32_t lower = 0;
 #pragma unroll
         for (int v = 0; v < V; ++v) s[v] = 0;
 #pragma unroll
         for (int q = 0; q < R; ++q) {
-            const int k = rb + q;
-            if (k < re) {
-                const int jn = ci[k];
-                Vec<T, V>::ld(X + (f.slot0 + jn) * Cp + cv * V, nb[q]);
-                wnb[q] = wr ? wr[k] : static_cast<T>(1);
-                lower |= (jn < lo ? 1u : 0u) << q;
+            if (c.jn[q] >= 0) {
+                Vec<T, V>::ld(X + (f.slot0 + c.jn[q]) * Cp + cv * V, nb[q]);
+                lower |= (c.jn[q] < lo ? 1u : 0u) << q;
             } else {
 #pragma unroll
                 for (int v = 0; v < V; ++v) nb[q][v] = 0;
-                wnb[q] = 0;
             }
 #pragma unroll
-            for (int v = 0; v < V; ++v) s[v] += wnb[q] * nb[q][v];
+            for (int v = 0; v < V; ++v) s[v] += c.wnb[q] * nb[q][v];
         }
         for (int k = rb + R; k < re; ++k) {  // rows longer than R
             T xv[V];
@@ -369,12 +424,9 @@ __device__ void csr_tile(const StepArgs &a, const FieldDev &f, const Tile &t, Si
             for (int v = 0; v < V; ++v) s[v] += wv * xv[v];
         }
         const int64_t self = f.slot0 + pos;
-        const T yv = Y[self];
-        const T d = DEG[f.csr0 + pos];
-        const uint32_t site = static_cast<uint32_t>(a.perm[f.csr0 + pos]);
-        const int mtr = MODEL == kModelBinomial ? a.trials[self] : 0;
-        finish_site<T, V, R, MODEL>(a, cx, X + self * Cp + cv * V, MEAN + self * Cp + cv * V, M2 + self * Cp + cv * V, yv,
-                                    mtr, d, site, sweep, f.stream, static_cast<uint32_t>(cv * V), s, nb, lower, wnb);
+        finish_site<T, V, R, MODEL>(a, cx, X + self * Cp + cv * V, MEAN + self * Cp + cv * V, M2 + self * Cp + cv * V, c.yv,
+                                    c.mtr, c.d, c.site, sweep, f.stream, static_cast<uint32_t>(cv * V), s, nb, lower, c.wnb,
+                                    c.drawn && c.sweep == sweep ? c.z : nullptr);
         if (re - rb > R) {
             // the lower-colour edges beyond the first R
             T xn[V], e2[V];
@@ -404,9 +456,12 @@ __device__ void csr_tile(const StepArgs &a, const FieldDev &f, const Tile &t, Si
 template <typename T, int V, int KIND, int MODEL>
 __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? (KIND == kCsr ? 2 : 3) : 1) colour_step_kernel(const StepArgs a)
 {
-    pdl_wait_then_release();
+    // Tiles and fields are never written by a sweep: read before the dependency wait.
     const Tile t = a.tiles[blockIdx.x];
     const FieldDev f = a.fields[t.field];
+    CsrSite<T, V> ahead;
+    if constexpr (KIND == kCsr) csr_ahead<T, V, MODEL>(a, f, t, ahead);
+    pdl_wait_then_release();
     const int CV = a.Cp / V;
     const int cv = threadIdx.x % CV;  // fixed per thread: kBlock is a multiple of CV
     const long long sweep_ll = a.ctl->sweep;
@@ -448,7 +503,7 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? (KIND == kCsr ? 2 : 3
     if constexpr (KIND == kLat2D4) lattice_parity_tile<T, V, false, MODEL>(a, f, t, cx, CV, cv_shift, sweep);
     else if constexpr (KIND == kLat3D6) lattice_parity_tile<T, V, true, MODEL>(a, f, t, cx, CV, cv_shift, sweep);
     else if constexpr (KIND == kLat2D8) lattice8_tile<T, V, MODEL>(a, f, t, cx, CV, cv_shift, sweep);
-    else csr_tile<T, V, MODEL>(a, f, t, cx, CV, cv_shift, sweep);
+    else csr_tile<T, V, MODEL>(a, f, t, cx, CV, cv_shift, sweep, ahead);
 
     // Deterministic block reduction of the 3 V partial sums of each chain in the state precision:
     // a shuffle tree over the lanes that share a chain vector (lanes equal mod CV), then the
