@@ -133,6 +133,18 @@ int gmrf::record_error(int st, const char *msg)
     return st;
 }
 
+// Small results on their way to the host, in pinned memory: a copy into it is one asynchronous
+// transfer (a copy into pageable memory waits for the stream twice), so a call that reads several
+// waits once.  Fields of up to kMailSites sites take their arrays through it too.
+constexpr int64_t kMailSites = 8192;
+struct HostMail {
+    SweepCtl ctl;
+    double now[2];
+    unsigned int flag;
+    double trace[2][kMailSites];
+    double site[3][kMailSites];
+};
+
 struct gmrf_sampler {
     int device = 0;
     cudaStream_t stream = nullptr;
@@ -190,6 +202,7 @@ struct gmrf_sampler {
     Part3 *partials = nullptr;
     double *trace_tau = nullptr, *trace_sig = nullptr, *trace_beta = nullptr;
     SweepCtl *ctl = nullptr;
+    HostMail *mail = nullptr;   // pinned: what a call reads back
     double *gpre = nullptr;     // [gpre_batch][F * Cp][4] precomputed variates of a batch
     int32_t gpre_batch = 0;     // sweeps per batch of precomputed variates
     double *staging = nullptr;  // [max_n] doubles for fetch
@@ -265,6 +278,8 @@ struct gmrf_sampler {
                 }
         for (void *p : allocs) cudaFree(p);
         allocs.clear();
+        if (mail) cudaFreeHost(mail);
+        mail = nullptr;
         if (capture_stream) cudaStreamDestroy(capture_stream);
         capture_stream = nullptr;
         if (side_stream) cudaStreamDestroy(side_stream);
@@ -1178,6 +1193,26 @@ gmrf_status poison(gmrf_sampler *s, cudaError_t e, const char *where)
     return cuda_status(CudaFail{e, where});
 }
 
+// The sweep control block, once everything enqueued before is done.
+cudaError_t read_ctl(gmrf_sampler *s, SweepCtl &c)
+{
+    cudaError_t e = cudaMemcpyAsync(&s->mail->ctl, s->ctl, sizeof(SweepCtl), cudaMemcpyDeviceToHost, s->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
+    if (e == cudaSuccess) c = s->mail->ctl;
+    return e;
+}
+
+// The last m values of a trace ring (cap values, sweep number `sweep` next), oldest first, into dst
+// (enqueued: at most two pieces of the ring).
+cudaError_t copy_trace(gmrf_sampler *s, double *dst, const double *ring, int64_t cap, int64_t sweep, int64_t m)
+{
+    const int64_t first = (sweep - m) % cap, head = std::min(m, cap - first);
+    cudaError_t e = cudaMemcpyAsync(dst, ring + first, sizeof(double) * head, cudaMemcpyDeviceToHost, s->stream);
+    if (e == cudaSuccess && m > head)
+        e = cudaMemcpyAsync(dst + head, ring, sizeof(double) * (m - head), cudaMemcpyDeviceToHost, s->stream);
+    return e;
+}
+
 // A bounded device wait that gave up (counted in the sweep control block) makes the results since
 // invalid: the call reports it and the sampler is poisoned.
 gmrf_status check_waits(gmrf_sampler *s, const SweepCtl &c)
@@ -1962,6 +1997,7 @@ gmrf_status gmrf_sampler_create(gmrf_sampler **out, const gmrf_field_desc *field
         CK(cudaGetDevice(&s->device));
         CK(cudaStreamCreateWithFlags(&s->capture_stream, cudaStreamNonBlocking));
         CK(s->alloc_t(&s->ctl, 1, sizeof(SweepCtl)));
+        CK(cudaMallocHost(reinterpret_cast<void **>(&s->mail), sizeof(HostMail)));
         SweepCtl c0{};
         c0.sweep = opts->start_sweep;
         CK(cudaMemcpyAsync(s->ctl, &c0, sizeof(c0), cudaMemcpyHostToDevice, s->stream));
@@ -2064,12 +2100,18 @@ gmrf_status gmrf_fetch_samples(gmrf_sampler *s, int32_t field, int32_t chain, do
     const int64_t n = h.n;
     try {
         SweepCtl c{};
-        CK(cudaMemcpyAsync(&c, s->ctl, sizeof(c), cudaMemcpyDeviceToHost, s->stream));
-        CK(cudaStreamSynchronize(s->stream));
+        CK(read_ctl(s, c));
         if (const gmrf_status w = check_waits(s, c)) return w;
         const bool plain = s->algorithm == GMRF_ALGO_PLAIN;
         const int64_t k = plain ? 0 : c.acc_count;
-        auto fetch = [&](const void *src, const void *m2, double scale, double *dst) {
+        // Small arrays go through the pinned mail and are handed on after one wait; larger ones
+        // straight to the caller (the stream orders the staging area's uses).
+        const bool mailed = n <= kMailSites;
+        double *const *to[3] = {&x_last, &x_mean, &x_var};
+        bool fetched[3] = {false, false, false};
+        auto fetch = [&](int slot, const void *src, const void *m2, double scale) {
+            double *dst = mailed ? s->mail->site[slot] : *to[slot];
+            fetched[slot] = true;
             if (plain) {
                 CK(cudaMemcpyAsync(dst, s->plain.x + chain * n, sizeof(double) * n, cudaMemcpyDeviceToHost, s->stream));
                 return;
@@ -2077,38 +2119,37 @@ gmrf_status gmrf_fetch_samples(gmrf_sampler *s, int32_t field, int32_t chain, do
             CK(launch_unpack(s->precision, s->fields_dev, s->fd[field], field, s->Cp, chain, src, m2, scale, s->perm_inv,
                              s->staging, s->stream));
             CK(cudaMemcpyAsync(dst, s->staging, sizeof(double) * n, cudaMemcpyDeviceToHost, s->stream));
-            CK(cudaStreamSynchronize(s->stream));
         };
         // Fused fields keep the state at the start of sweep t in buffer t & 1.
         void *xcur = (h.fused && (c.sweep & 1)) ? s->x_alt : s->x;
-        if (x_last) fetch(xcur, nullptr, 1.0, x_last);
+        if (x_last) fetch(0, xcur, nullptr, 1.0);
         if (x_mean) {
             if (plain || k < 1) std::fill(x_mean, x_mean + n, plain ? NAN : 0.0);
-            else fetch(s->mean, nullptr, 1.0, x_mean);
+            else fetch(1, s->mean, nullptr, 1.0);
         }
         if (x_var) {
             if (plain || k < 2) std::fill(x_var, x_var + n, NAN);
-            else fetch(nullptr, s->m2, 1.0 / static_cast<double>(k - 1), x_var);
+            else fetch(2, nullptr, s->m2, 1.0 / static_cast<double>(k - 1));
         }
         const int64_t cap = s->opts.trace_capacity;
         const int64_t avail = std::min<int64_t>(c.sweep - s->opts.start_sweep, cap);
         if (n_trace) *n_trace = avail;
         const int64_t hc = plain ? chain : static_cast<int64_t>(field) * s->Cp + chain;
-        if ((tau_trace || sigma2_trace) && trace_cap > 0 && avail > 0) {
-            std::vector<double> rt(static_cast<size_t>(cap)), rs(static_cast<size_t>(cap));
-            CK(cudaMemcpyAsync(rt.data(), s->trace_tau + hc * cap, sizeof(double) * cap, cudaMemcpyDeviceToHost, s->stream));
-            CK(cudaMemcpyAsync(rs.data(), s->trace_sig + hc * cap, sizeof(double) * cap, cudaMemcpyDeviceToHost, s->stream));
-            CK(cudaStreamSynchronize(s->stream));
-            const int64_t m = std::min(trace_cap, avail);
-            for (int64_t q = 0; q < m; ++q) {
-                const int64_t sw = c.sweep - m + q;
-                if (tau_trace) tau_trace[q] = rt[sw % cap];
-                if (sigma2_trace) sigma2_trace[q] = rs[sw % cap];
-            }
-        }
-        if (tau_now) CK(cudaMemcpyAsync(tau_now, s->tau + hc, sizeof(double), cudaMemcpyDeviceToHost, s->stream));
-        if (sigma2_now) CK(cudaMemcpyAsync(sigma2_now, s->sig2 + hc, sizeof(double), cudaMemcpyDeviceToHost, s->stream));
+        const int64_t m = std::min(trace_cap, avail);
+        double *traces[2] = {tau_trace, sigma2_trace};
+        const double *rings[2] = {s->trace_tau, s->trace_sig};
+        for (int q = 0; q < 2; ++q)
+            if (traces[q] && m > 0)
+                CK(copy_trace(s, m <= kMailSites ? s->mail->trace[q] : traces[q], rings[q] + hc * cap, cap, c.sweep, m));
+        if (tau_now) CK(cudaMemcpyAsync(&s->mail->now[0], s->tau + hc, sizeof(double), cudaMemcpyDeviceToHost, s->stream));
+        if (sigma2_now) CK(cudaMemcpyAsync(&s->mail->now[1], s->sig2 + hc, sizeof(double), cudaMemcpyDeviceToHost, s->stream));
         CK(cudaStreamSynchronize(s->stream));
+        for (int q = 0; q < 3; ++q)
+            if (mailed && fetched[q]) std::copy(s->mail->site[q], s->mail->site[q] + n, *to[q]);
+        for (int q = 0; q < 2; ++q)
+            if (traces[q] && m > 0 && m <= kMailSites) std::copy(s->mail->trace[q], s->mail->trace[q] + m, traces[q]);
+        if (tau_now) *tau_now = s->mail->now[0];
+        if (sigma2_now) *sigma2_now = s->mail->now[1];
     } catch (const CudaFail &f) {
         s->poisoned = true;
         return cuda_status(f);
@@ -2126,22 +2167,20 @@ gmrf_status gmrf_fetch_pooled(gmrf_sampler *s, int32_t field, double *mean, doub
     if (s->algorithm == GMRF_ALGO_PLAIN) return fail(GMRF_E_UNSUPPORTED, "the plain sweep keeps no running moments");
     const int64_t n = s->hf[field].n;
     try {
-        SweepCtl c{};
-        CK(cudaMemcpyAsync(&c, s->ctl, sizeof(c), cudaMemcpyDeviceToHost, s->stream));
-        CK(cudaStreamSynchronize(s->stream));
-        if (const gmrf_status w = check_waits(s, c)) return w;
-        const int64_t k = c.acc_count;
-        if (mean && k < 1) std::fill(mean, mean + n, 0.0);
-        if (var && s->C * k < 2) std::fill(var, var + n, NAN);
-        double *dm = (mean && k >= 1) ? s->staging : nullptr;
-        double *dv = (var && s->C * k >= 2) ? s->pool_stage : nullptr;
-        if (dm || dv) {
-            CK(launch_pool(s->precision, s->fields_dev, s->fd[field], field, s->Cp, s->C, k, s->mean, s->m2,
+        // The pooling kernel takes the number of accumulated sweeps from the control block (0 and NaN
+        // where there are too few), so the call waits once.
+        const bool mailed = n <= kMailSites;
+        double *dm = mean ? s->staging : nullptr, *dv = var ? s->pool_stage : nullptr;
+        if (dm || dv)
+            CK(launch_pool(s->precision, s->fields_dev, s->fd[field], field, s->Cp, s->C, s->ctl, s->mean, s->m2,
                            s->perm_inv, dm, dv, s->stream));
-            if (dm) CK(cudaMemcpyAsync(mean, dm, sizeof(double) * n, cudaMemcpyDeviceToHost, s->stream));
-            if (dv) CK(cudaMemcpyAsync(var, dv, sizeof(double) * n, cudaMemcpyDeviceToHost, s->stream));
-            CK(cudaStreamSynchronize(s->stream));
-        }
+        if (dm) CK(cudaMemcpyAsync(mailed ? s->mail->site[0] : mean, dm, sizeof(double) * n, cudaMemcpyDeviceToHost, s->stream));
+        if (dv) CK(cudaMemcpyAsync(mailed ? s->mail->site[1] : var, dv, sizeof(double) * n, cudaMemcpyDeviceToHost, s->stream));
+        SweepCtl c{};
+        CK(read_ctl(s, c));
+        if (const gmrf_status w = check_waits(s, c)) return w;
+        if (mailed && dm) std::copy(s->mail->site[0], s->mail->site[0] + n, mean);
+        if (mailed && dv) std::copy(s->mail->site[1], s->mail->site[1] + n, var);
     } catch (const CudaFail &f) {
         s->poisoned = true;
         return cuda_status(f);
@@ -2162,22 +2201,24 @@ gmrf_status gmrf_fetch_intercept(gmrf_sampler *s, int32_t field, int32_t chain, 
     if (trace_cap < 0) return fail(GMRF_E_INVALID, "trace_cap must be >= 0");
     try {
         SweepCtl c{};
-        CK(cudaMemcpyAsync(&c, s->ctl, sizeof(c), cudaMemcpyDeviceToHost, s->stream));
-        CK(cudaStreamSynchronize(s->stream));
+        CK(read_ctl(s, c));
         if (const gmrf_status w = check_waits(s, c)) return w;
         const int64_t cap = s->opts.trace_capacity;
         const int64_t avail = std::min<int64_t>(c.sweep - s->opts.start_sweep, cap);
         if (n_trace) *n_trace = avail;
         const int64_t hc = static_cast<int64_t>(field) * s->Cp + chain;
         if (beta0_trace && trace_cap > 0 && avail > 0) {
-            std::vector<double> rb(static_cast<size_t>(cap));
-            CK(cudaMemcpyAsync(rb.data(), s->trace_beta + hc * cap, sizeof(double) * cap, cudaMemcpyDeviceToHost, s->stream));
-            CK(cudaStreamSynchronize(s->stream));
             const int64_t m = std::min(trace_cap, avail);
-            for (int64_t q = 0; q < m; ++q) beta0_trace[q] = rb[(c.sweep - m + q) % cap];
+            const bool mailed = m <= kMailSites;
+            CK(copy_trace(s, mailed ? s->mail->trace[0] : beta0_trace, s->trace_beta + hc * cap, cap, c.sweep, m));
+            if (mailed) {
+                CK(cudaStreamSynchronize(s->stream));
+                std::copy(s->mail->trace[0], s->mail->trace[0] + m, beta0_trace);
+            }
         }
-        if (beta0_now) CK(cudaMemcpyAsync(beta0_now, s->beta + hc, sizeof(double), cudaMemcpyDeviceToHost, s->stream));
+        if (beta0_now) CK(cudaMemcpyAsync(&s->mail->now[0], s->beta + hc, sizeof(double), cudaMemcpyDeviceToHost, s->stream));
         CK(cudaStreamSynchronize(s->stream));
+        if (beta0_now) *beta0_now = s->mail->now[0];
     } catch (const CudaFail &f) {
         s->poisoned = true;
         return cuda_status(f);
@@ -2199,8 +2240,7 @@ gmrf_status gmrf_trace_diagnostics(gmrf_sampler *s, int32_t field, int32_t param
     if (n_last < 0) return fail(GMRF_E_INVALID, "n_last must be >= 0");
     try {
         SweepCtl c{};
-        CK(cudaMemcpyAsync(&c, s->ctl, sizeof(c), cudaMemcpyDeviceToHost, s->stream));
-        CK(cudaStreamSynchronize(s->stream));
+        CK(read_ctl(s, c));
         if (const gmrf_status w = check_waits(s, c)) return w;
         const int64_t cap = s->opts.trace_capacity;
         const int64_t avail = std::min<int64_t>(c.sweep - s->opts.start_sweep, cap);
@@ -2246,8 +2286,7 @@ gmrf_status gmrf_site_psrf(gmrf_sampler *s, int32_t field, double *psrf, double 
     if (s->C < 2) return fail(GMRF_E_INVALID, "the PSRF needs at least 2 chains");
     try {
         SweepCtl c{};
-        CK(cudaMemcpyAsync(&c, s->ctl, sizeof(c), cudaMemcpyDeviceToHost, s->stream));
-        CK(cudaStreamSynchronize(s->stream));
+        CK(read_ctl(s, c));
         if (const gmrf_status w = check_waits(s, c)) return w;
         if (c.acc_count < 2) return fail(GMRF_E_INVALID, "the PSRF needs at least 2 accumulated sweeps");
         unsigned long long *mx = reinterpret_cast<unsigned long long *>(s->diag_out + static_cast<int64_t>(s->Cp) * 4 + 1);
@@ -2314,6 +2353,7 @@ gmrf_status gmrf_sampler_set_data(gmrf_sampler *s, int32_t field, const double *
         for (const HostField &h : s->hf) max_n = std::max<int64_t>(max_n, h.n);
         cudaError_t e = s->alloc_t(&s->data_stage, static_cast<size_t>(max_n) * (1 + s->C), sizeof(double));
         if (e == cudaSuccess) e = s->alloc_t(&s->data_flag, 1, sizeof(unsigned int));
+        if (e == cudaSuccess) e = cudaMemsetAsync(s->data_flag, 0, sizeof(unsigned int), s->stream);
         if (e == cudaSuccess && binomial)
             e = s->alloc_t(&s->trials_stage, static_cast<size_t>(max_n), sizeof(int32_t));
         if (e != cudaSuccess) {
@@ -2339,10 +2379,11 @@ gmrf_status gmrf_sampler_set_data(gmrf_sampler *s, int32_t field, const double *
                                    cudaMemcpyHostToDevice, s->stream));
             CK(launch_check_data(y_d, binomial ? s->trials_stage : nullptr, x0 ? x0_d : nullptr, n,
                                  x0 ? n * s->C : 0, s->data_flag, s->stream));
-            unsigned int bad = 0;
-            CK(cudaMemcpyAsync(&bad, s->data_flag, sizeof(bad), cudaMemcpyDeviceToHost, s->stream));
+            CK(cudaMemcpyAsync(&s->mail->flag, s->data_flag, sizeof(unsigned int), cudaMemcpyDeviceToHost, s->stream));
             CK(cudaStreamSynchronize(s->stream));  // the host arrays may be reused from here on
             // only the staging buffer was written
+            const unsigned int bad = s->mail->flag;
+            if (bad) CK(cudaMemsetAsync(s->data_flag, 0, sizeof(unsigned int), s->stream));
             if (bad & 1u) return fail(GMRF_E_INVALID, "y must be finite");
             if (bad & 2u) return fail(GMRF_E_INVALID, "trials must be in 0..4095");
             if (bad & 4u) return fail(GMRF_E_INVALID, "successes y must be in [0, trials]");
@@ -2401,8 +2442,7 @@ gmrf_status gmrf_sampler_info(gmrf_sampler *s, gmrf_info *out)
     if (s->poisoned) return fail(GMRF_E_STATE, "sampler is poisoned by an earlier CUDA error");
     if (const gmrf_status r = restart_if_pending(s)) return r;
     SweepCtl c{};
-    cudaError_t e = cudaMemcpyAsync(&c, s->ctl, sizeof(c), cudaMemcpyDeviceToHost, s->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
+    cudaError_t e = read_ctl(s, c);
     if (e != cudaSuccess) return poison(s, e, "info");
     if (const gmrf_status w = check_waits(s, c)) return w;
     out->nfields = s->nfields;

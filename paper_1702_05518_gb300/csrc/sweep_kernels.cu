@@ -805,7 +805,7 @@ __device__ __forceinline__ double divide(double a, const Divisor &v)
 
 // Running moments pooled over the C chains of one field, natural order, FP64: mean = the chains'
 // means averaged; var = the sum over chains of M2_c + k (mean_c - mean)^2, over C k - 1 (the
-// variance of all C k draws).  k >= 1 accumulated draws per chain.  CP: the layout's chains when
+// variance of all C k draws); 0 and NaN where k accumulated draws per chain are too few.  CP: the layout's chains when
 // 1, 2, 4 or 8 (a site's values are loaded as vectors and kept in registers), else 0.
 //
 // Bound by the FP64 pipe (measured: about one lane per clock and SM): four FP64 operations per
@@ -815,13 +815,14 @@ __device__ __forceinline__ double divide(double a, const Divisor &v)
 // the conversions to integer operations changed nothing).
 template <typename T, int CP>
 __global__ void __launch_bounds__(256) pool_kernel(const FieldDev *fields, int32_t fidx, int32_t Cp_, int32_t C,
-                                                   int64_t k, const T *mean, const T *m2, const int32_t *perm_inv,
+                                                   const SweepCtl *ctl, const T *mean, const T *m2, const int32_t *perm_inv,
                                                    double *out_mean, double *out_var)
 {
     const FieldDev f = fields[fidx];
     const int Cp = CP ? CP : Cp_;
     constexpr int V = CP == 0 ? 1 : (sizeof(T) == 8 ? (CP < 2 ? CP : 2) : (CP < 4 ? CP : 4));
     constexpr int NR = CP ? CP : 1;
+    const int64_t k = ctl->acc_count;
     const double kd = static_cast<double>(k);
     const Divisor by_c{static_cast<double>(C), 1.0 / static_cast<double>(C)};
     const double dof = static_cast<double>(C * k - 1);
@@ -867,8 +868,8 @@ __global__ void __launch_bounds__(256) pool_kernel(const FieldDev *fields, int32
                     ss += static_cast<double>(qp[c]);
                 }
         }
-        if (out_mean) out_mean[i] = mu;
-        if (out_var) out_var[i] = divide(fma(kd, dd, ss), by_dof);
+        if (out_mean) out_mean[i] = k < 1 ? 0.0 : mu;
+        if (out_var) out_var[i] = C * k < 2 ? __longlong_as_double(0x7ff8000000000000ll) : divide(fma(kd, dd, ss), by_dof);
     }
 }
 
@@ -1021,8 +1022,6 @@ __global__ void check_data_kernel(const double *y, const int32_t *trials, const 
 cudaError_t launch_check_data(const double *y, const int32_t *trials, const double *x0, int64_t n, int64_t nx0,
                               unsigned int *flag, cudaStream_t stream)
 {
-    cudaError_t e = cudaMemsetAsync(flag, 0, sizeof(unsigned int), stream);
-    if (e != cudaSuccess) return e;
     check_data_kernel<<<grid_for(n > nx0 ? n : nx0, 256), 256, 0, stream>>>(y, trials, x0, n, nx0, flag);
     return cudaGetLastError();
 }
@@ -1049,12 +1048,12 @@ cudaError_t launch_unpack(int precision, const FieldDev *fields_dev, const Field
 }
 
 cudaError_t launch_pool(int precision, const FieldDev *fields_dev, const FieldDev &f, int32_t fidx, int32_t Cp,
-                        int32_t C, int64_t k, const void *mean, const void *m2, const int32_t *perm_inv,
+                        int32_t C, const SweepCtl *ctl, const void *mean, const void *m2, const int32_t *perm_inv,
                         double *out_mean, double *out_var, cudaStream_t stream)
 {
     const int grid = grid_for(f.n, 256);
     auto go = [&](auto *kernel, auto *me, auto *q) {
-        kernel<<<grid, 256, 0, stream>>>(fields_dev, fidx, Cp, C, k, me, q, perm_inv, out_mean, out_var);
+        kernel<<<grid, 256, 0, stream>>>(fields_dev, fidx, Cp, C, ctl, me, q, perm_inv, out_mean, out_var);
     };
     auto pick = [&](auto *me, auto *q) {
         using T = std::remove_cv_t<std::remove_pointer_t<decltype(me)>>;
