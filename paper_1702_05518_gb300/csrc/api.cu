@@ -719,7 +719,7 @@ cudaError_t plan_tile_resident(gmrf_sampler *s)
         const int zrows = march_ahead_rows(s->Cp, rows);
         cudaError_t em = plan_march_grid(kind, s->Cp, s->mtile_cnt[kind], zrows, &fits);
         if (em == cudaSuccess && fits)
-            em = s->alloc_t(&s->res_pm, static_cast<size_t>(3) * s->Cp * s->mtile_cnt[kind], sizeof(double));
+            em = s->alloc_t(&s->res_pm, static_cast<size_t>(2) * 3 * s->Cp * s->mtile_cnt[kind], sizeof(double));
         if (em != cudaSuccess || !fits) return em;
         s->march_grid = true;
         s->march_zrows = zrows;
@@ -759,7 +759,7 @@ cudaError_t plan_grid(gmrf_sampler *s, const std::vector<int32_t> &coff0)
     }
     if (e != cudaSuccess || !s->grid_blocks) return e;
     s->res_batch = std::min(128, std::max(64, s->opts.graph_sweeps));
-    return s->alloc_t(&s->res_pm, static_cast<size_t>(3) * s->Cp * s->grid_blocks, sizeof(double));
+    return s->alloc_t(&s->res_pm, static_cast<size_t>(2) * 3 * s->Cp * s->grid_blocks, sizeof(double));
 }
 
 // The resident path applies to a single fused 2-D lattice field with the Gaussian likelihood whose

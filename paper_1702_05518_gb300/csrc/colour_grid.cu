@@ -172,12 +172,13 @@ __global__ void __launch_bounds__(kGridThreads, 1) csr_grid_kernel(const GridSwe
             aR[v] = 0.0f;
             aA[v] = 0.0f;
         }
+        double *const pm = ra.pm + (it & 1) * 3 * Cp * nblk;  // (a graph of one colour has one barrier per sweep)
         for (int c = 0; c < K; ++c) {
             for (int q = tid; (q >> cvs) < cnt; q += kGridThreads) {
                 if (q != tid) fetch(lo + (q >> cvs), sw, acc);  // beyond one position per thread
                 update(coffs[c], acc, inv_k);
             }
-            if (c + 1 == K) grid_partials<V, kGridThreads>(aS, aR, aA, CV, Cp, red, ra.pm, nblk);
+            if (c + 1 == K) grid_partials<V, kGridThreads>(aS, aR, aA, CV, Cp, red, pm, nblk);
             __syncthreads();  // the block's stores of this step
             if (tid == 0) grid_arrive(a.ctl);
             arrivals += nblk;
@@ -194,7 +195,7 @@ __global__ void __launch_bounds__(kGridThreads, 1) csr_grid_kernel(const GridSwe
         if (sh.abort) break;
         if (acc) ++acc_count;
         acc = acc_next;
-        grid_draw(sh, h, ra.pm, nblk, f, sw, it, blockIdx.x == 0);
+        grid_draw(sh, h, pm, nblk, f, sw, it, blockIdx.x == 0);
         __syncthreads();
     }
     grid_finish(a.ctl, sweep0 + ra.count, acc_count);
@@ -422,6 +423,7 @@ __global__ void __launch_bounds__(kGridThreads, 1) lattice3d_grid_kernel(const G
             aA[v] = 0.0f;
         }
         __syncthreads();
+        double *const pm = ra.pm + (it & 1) * 3 * CP * nblk;
 #pragma unroll 1
         for (int c = 0; c < 2; ++c) {
 #pragma unroll
@@ -432,7 +434,7 @@ __global__ void __launch_bounds__(kGridThreads, 1) lattice3d_grid_kernel(const G
 #pragma unroll
                 for (int u = 0; u < UB; ++u) update(t[u], m0 + u, c);
             }
-            if (c == 1) grid_partials<V, kGridThreads>(aS, aR, aA, CV, CP, red, ra.pm, nblk);
+            if (c == 1) grid_partials<V, kGridThreads>(aS, aR, aA, CV, CP, red, pm, nblk);
             __syncthreads();  // the block's stores of this step
             if (tid == 0) grid_arrive(a.ctl);
             arrivals += nblk;
@@ -443,7 +445,7 @@ __global__ void __launch_bounds__(kGridThreads, 1) lattice3d_grid_kernel(const G
         }
         if (sh.abort) break;
         if (acc) ++acc_count;
-        grid_draw(sh, h, ra.pm, nblk, f, sw, it, blockIdx.x == 0);
+        grid_draw(sh, h, pm, nblk, f, sw, it, blockIdx.x == 0);
         __syncthreads();
     }
     grid_finish(a.ctl, sweep0 + ra.count, acc_count);

@@ -340,7 +340,7 @@ struct GridSweepArgs {
     StepArgs s;               // the field's buffers (update 1; tiles unused)
     HyperArgs h;              // the conjugate draws at the end of each sweep (end_of_sweep 1)
     int32_t count;            // sweeps of the launch
-    double *pm;               // [Cp][S, R, A][block] the blocks' partial sums
+    double *pm;               // [sweep's parity][Cp][S, R, A][block] the blocks' partial sums
     uint32_t extra_arrivals;  // 0; 1 under GMRF_FLAG_TEST_STALL (no grid barrier completes)
     uint64_t wait_ns;         // limit of a wait at the grid barrier
     uint32_t u_m;             // 3-D lattices: invariant-divisor constants of the units in a row
@@ -375,7 +375,7 @@ struct MarchArgs {
     HyperArgs h;
     int32_t count;
     int32_t zrows;            // rows of a chunk whose normals are drawn ahead
-    double *pm;               // [Cp][S, R, A][block]
+    double *pm;               // [sweep's parity][Cp][S, R, A][block]
     uint32_t extra_arrivals;
     uint64_t wait_ns;
 };

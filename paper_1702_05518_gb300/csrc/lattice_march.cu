@@ -684,7 +684,10 @@ __global__ void __launch_bounds__(kMarchThreads, 1) march_grid_kernel(const Marc
         if (m.active()) m.march();
         if (acc) ++acc_count;
         const float s = march_sums<V>(m.aS, m.aR, m.aA, red);
-        if (tid < V * 3) a.pm[tid * nblk + blockIdx.x] = static_cast<double>(s);  // [chain][S, R, A][block]
+        // [chain][S, R, A][block], by the sweep's parity: a block of a few rows ends its next sweep while
+        // others, still drawing ahead, have not read this one's sums
+        double *const pm = a.pm + (it & 1) * 3 * V * nblk;
+        if (tid < V * 3) pm[tid * nblk + blockIdx.x] = static_cast<double>(s);
         __syncthreads();  // the block's stores of this sweep
         if (tid == 0) grid_arrive(ctl);
         arrivals += nblk;
@@ -692,7 +695,7 @@ __global__ void __launch_bounds__(kMarchThreads, 1) march_grid_kernel(const Marc
         if (tid == 0 && grid_wait(ctl, arrivals, a.wait_ns)) sh.abort = 1;
         __syncthreads();
         if (sh.abort) break;
-        grid_draw(sh, h, a.pm, nblk, f, sw, it, blockIdx.x == 0);
+        grid_draw(sh, h, pm, nblk, f, sw, it, blockIdx.x == 0);
         __syncthreads();
     }
     grid_finish(ctl, sweep0 + a.count, acc_count);

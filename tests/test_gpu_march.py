@@ -3,7 +3,10 @@ launch per sweep or a batch of sweeps per cooperative launch.  Parity with the o
 one sweep, 1e-4 on states, means and traces after more) where the decomposition can go wrong: widths
 around a strip's columns and their halo, row lengths of every offset to the Philox blocks, chunk ends of
 both parities, images of a row or a column, one to sixteen chains; several fields in one sampler; the
-sums of an extra draw.  (That the two forms agree bit for bit: test_gpu_fused_resident.py.)
+sums of an extra draw.  The two forms agree bit for bit.
+
+Single fields of one wave of tiles take the tiled kernels by default; asking for the chains per thread
+the sampler would choose anyway sends them to the marching warps.
 """
 import numpy as np
 import pytest
@@ -22,9 +25,13 @@ def _built():
     build.build()
 
 
-# A strip owns 120 columns (one or two chains), 60 or 56 (more); chunks of a few rows.
+# A strip owns 120 columns (one chain), 60 or 56 (two; 4 and 8 neighbours); chunks of a few rows.
 DIMS = [(1, 1), (1, 130), (9, 1), (2, 3), (5, 2), (7, 119), (8, 120), (9, 121), (6, 122), (11, 123), (13, 125), (4, 240),
         (33, 241), (10, 57), (17, 61), (12, 113), (40, 118), (67, 66), (131, 35)]
+
+
+def _march(chains):
+    return {"tuning": {"chains_per_thread": chains}} if chains <= 2 else {}
 
 
 def _run(fields, chains, calls, extra=False, **kw):
@@ -56,10 +63,10 @@ def _check(f, res, chains, T, tol, stream=0, **kw):
 def test_parity_with_the_oracle(kind, dims, chains):
     # (single-chain 8-neighbour rows of a multiple of four take the quad kernel)
     f = wl.small_lattice(kind, dims, 9)
-    one, _ = _run([f], chains, [1], flags=g.FLAG_NO_RESIDENT)
+    one, _ = _run([f], chains, [1], flags=g.FLAG_NO_RESIDENT, **_march(chains))
     _check(f, one[0], chains, 1, TOL_FP32_1)
     kw = dict(prior=g.PRIOR_PCAR, rho=0.9) if chains != 2 else dict(intercept=True)
-    res, info = _run([f], chains, [23, 8], burn_in=11, flags=g.FLAG_NO_RESIDENT, graph_sweeps=5, **kw)
+    res, info = _run([f], chains, [23, 8], burn_in=11, flags=g.FLAG_NO_RESIDENT, graph_sweeps=5, **kw, **_march(chains))
     assert info["accumulated"] == 20
     kw = dict(prior="pcar", rho=0.9) if chains != 2 else dict(intercept=True)
     _check(f, res[0], chains, 31, TOL_FP32_1000, burn_in=11, **kw)
@@ -72,9 +79,22 @@ def test_parity_with_the_oracle(kind, dims, chains):
 def test_batches_of_sweeps_parity(kind, dims, chains):
     f = wl.small_lattice(kind, dims, 10)
     T = 6 if dims[0] >= 700 else 40
-    res, info = _run([f], chains, [T], burn_in=T // 2, graph_sweeps=16)
+    res, info = _run([f], chains, [T], burn_in=T // 2, graph_sweeps=16, **_march(chains))
     assert info["wait_timeouts"] == 0
     _check(f, res[0], chains, T, TOL_FP32_1000, burn_in=T // 2)
+
+
+@pytest.mark.parametrize("kind,dims,chains", [(wl.LATTICE2D_4, (1500, 1999), 1), (wl.LATTICE2D_8, (901, 1510), 2),
+                                              (wl.LATTICE2D_4, (41, 241), 1), (wl.LATTICE2D_8, (70, 123), 1),
+                                              (wl.LATTICE2D_8, (90, 61), 2)])
+def test_batches_equal_single_sweeps(kind, dims, chains):
+    f = wl.small_lattice(kind, dims, 14)
+    a, info = _run([f], chains, [7, 2], burn_in=3, **_march(chains))
+    assert info["resident"] == 0  # not the small-lattice or tile-resident form
+    b, _ = _run([f], chains, [7, 2], burn_in=3, flags=g.FLAG_NO_RESIDENT, **_march(chains))
+    for c in range(chains):
+        for k in ("x", "mean", "var", "tau_trace", "sigma2_trace"):
+            np.testing.assert_array_equal(a[0][c][k], b[0][c][k], err_msg=k)
 
 
 @pytest.mark.parametrize("chains", [1, 3])
@@ -94,7 +114,7 @@ def test_sums_of_an_extra_draw(kind, chains):
     # the draw after hyper_update uses the sums of the current state: the tiled kernel's agree
     f = wl.small_lattice(kind, (45, 131), 12)
     out = []
-    for tuning in (None, {"fused_rows": [16, 16], "fused_cols": [32, 32], "fused_threads": [512, 512]}):
+    for tuning in (_march(chains).get("tuning"), {"fused_rows": [16, 16], "fused_cols": [32, 32], "fused_threads": [512, 512]}):
         with g.Sampler([f], precision=g.FP32, chains=chains, seed=5, flags=g.FLAG_NO_RESIDENT, prior=g.PRIOR_PCAR, rho=0.8,
                        tuning=tuning) as s:
             s.sweep(4)
