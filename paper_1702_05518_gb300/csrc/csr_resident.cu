@@ -466,12 +466,11 @@ cudaError_t launch_cl(int chains, const ResCsrArgs &a, size_t smem, cudaStream_t
 template <typename T, int MP>
 cudaError_t prepare_mp(size_t smem)
 {
-    constexpr auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    cudaError_t e = cudaFuncSetAttribute(csr_resident_kernel<T, 1, MP>, attr, static_cast<int>(smem));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(csr_resident_kernel<T, 2, MP>, attr, static_cast<int>(smem));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(csr_resident_kernel<T, 4, MP>, attr, static_cast<int>(smem));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(csr_resident_kernel<T, 8, MP>, attr, static_cast<int>(smem));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(csr_resident_kernel<T, 16, MP>, attr, static_cast<int>(smem));
+    cudaError_t e = allow_smem(csr_resident_kernel<T, 1, MP>, smem);
+    if (e == cudaSuccess) e = allow_smem(csr_resident_kernel<T, 2, MP>, smem);
+    if (e == cudaSuccess) e = allow_smem(csr_resident_kernel<T, 4, MP>, smem);
+    if (e == cudaSuccess) e = allow_smem(csr_resident_kernel<T, 8, MP>, smem);
+    if (e == cudaSuccess) e = allow_smem(csr_resident_kernel<T, 16, MP>, smem);
     // clusters of 16 blocks exceed the portable size of 8
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(csr_resident_kernel<T, 16, MP>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);

@@ -439,4 +439,21 @@ struct PlainArgs {
 };
 cudaError_t launch_plain_sweep(const PlainArgs &a, cudaStream_t stream, int64_t *launches);
 
+// Let a kernel use all the shared memory that a block can have beside its static part.  The limit is
+// the kernel's and not a sampler's: one set to what one sampler needs fails the launches of another that
+// needs more.  An error if `smem` is beyond it.
+template <typename K>
+cudaError_t allow_smem(K *kernel, size_t smem)
+{
+    int dev = 0, most = 0;
+    cudaFuncAttributes fa;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, kernel);
+    if (e != cudaSuccess) return e;
+    const int limit = most - static_cast<int>(fa.sharedSizeBytes);
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                static_cast<int>(smem) > limit ? static_cast<int>(smem) : limit);
+}
+
 }  // namespace gmrf

@@ -787,14 +787,10 @@ cudaError_t launch_t(const FusedArgs &a, size_t smem, cudaStream_t stream)
 template <typename T, int V, int KIND>
 cudaError_t prepare_t(size_t smem)
 {
-    const int b = static_cast<int>(smem);
-    cudaError_t e = cudaFuncSetAttribute(lattice_fused_kernel<T, V, KIND, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(lattice_fused_kernel<T, V, KIND, 1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(lattice_fused_fast<T, KIND, 512, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(lattice_fused_fast<T, KIND, 1024, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
+    cudaError_t e = allow_smem(lattice_fused_kernel<T, V, KIND, 512>, smem);
+    if (e == cudaSuccess) e = allow_smem(lattice_fused_kernel<T, V, KIND, 1024>, smem);
+    if (e == cudaSuccess) e = allow_smem(lattice_fused_fast<T, KIND, 512, V>, smem);
+    if (e == cudaSuccess) e = allow_smem(lattice_fused_fast<T, KIND, 1024, V>, smem);
     return e;
 }
 

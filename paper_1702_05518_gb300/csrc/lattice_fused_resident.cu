@@ -505,8 +505,7 @@ cudaError_t lattice_fused_resident_fits(int kind, int threads, int Cp, size_t sm
     if (e != cudaSuccess) return e;
 #define GMRF_FR_FITS(KD, N, C)                                                                                  \
     if (kind == KD && threads == N && Cp == C) {                                                              \
-        e = cudaFuncSetAttribute(lattice_fused_resident<KD, N, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                                 static_cast<int>(smem));                                                     \
+        e = allow_smem(lattice_fused_resident<KD, N, C>, smem);                                                \
         if (e == cudaSuccess)                                                                                 \
             e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lattice_fused_resident<KD, N, C>, N, smem); \
         if (e != cudaSuccess) {                                                                               \

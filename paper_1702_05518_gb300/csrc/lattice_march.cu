@@ -813,8 +813,7 @@ cudaError_t plan_march_grid(int kind, int Cp, int blocks, int zrows, bool *fits)
             if (e == cudaSuccess)
                 e = with_march(kind, Cp, plain, [&](auto kd, auto v, auto pl) {
                     auto *k = march_grid_kernel<decltype(kd)::value, decltype(v)::value, decltype(pl)::value>;
-                    // the most any sampler asks for (the limit is the kernel's, not the sampler's)
-                    const cudaError_t a = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kAheadBytes);
+                    const cudaError_t a = allow_smem(k, z_row_bytes(Cp) * zrows);
                     int n = 0;
                     const cudaError_t o = a != cudaSuccess ? a : cudaOccupancyMaxActiveBlocksPerMultiprocessor(
                                                                      &n, k, kMarchThreads, z_row_bytes(Cp) * zrows);

@@ -621,8 +621,7 @@ cudaError_t prepare_lattice_quad(int qcs, int nt, int nq, size_t smem)
 {
 #define GMRF_QUAD_CFG(Q, N, M)                                                                                   \
     if (qcs == Q && nt == N && nq == M)                                                                       \
-        return cudaFuncSetAttribute(lattice_quad_kernel<Q, N, M>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                                    static_cast<int>(smem));
+        return allow_smem(lattice_quad_kernel<Q, N, M>, smem);
     GMRF_QUAD_CFG(64, 768, 3)
     GMRF_QUAD_CFG(64, 1024, 2)
     GMRF_QUAD_CFG(32, 1024, 2)
@@ -659,8 +658,7 @@ cudaError_t lattice_quad_resident_fits(int qcs, int nt, int nq, size_t smem, int
     if (e != cudaSuccess) return e;
 #define GMRF_QUAD_CFG(Q, N, M)                                                                                   \
     if (qcs == Q && nt == N && nq == M) {                                                                     \
-        e = cudaFuncSetAttribute(lattice_quad_resident_kernel<Q, N, M>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                                 static_cast<int>(smem));                                                     \
+        e = allow_smem(lattice_quad_resident_kernel<Q, N, M>, smem);                                      \
         if (e == cudaSuccess)                                                                                 \
             e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lattice_quad_resident_kernel<Q, N, M>, N, smem); \
         if (e != cudaSuccess) return e;                                                                       \

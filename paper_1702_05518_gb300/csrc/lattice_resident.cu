@@ -399,11 +399,9 @@ cudaError_t launch_ni(int NI, int threads, int chains, const ResidentArgs &a, si
 template <typename T, int KIND>
 cudaError_t prepare_ni(int NI, size_t smem)
 {
-    const int s = static_cast<int>(smem);
-    constexpr auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    if (NI == 1) return cudaFuncSetAttribute(lattice_resident_kernel<T, KIND, 1>, attr, s);
-    if (NI == 2 || KIND == kLat2D8) return cudaFuncSetAttribute(lattice_resident_kernel<T, KIND, 2>, attr, s);
-    return cudaFuncSetAttribute(lattice_resident_kernel<T, kLat2D4, 4>, attr, s);
+    if (NI == 1) return allow_smem(lattice_resident_kernel<T, KIND, 1>, smem);
+    if (NI == 2 || KIND == kLat2D8) return allow_smem(lattice_resident_kernel<T, KIND, 2>, smem);
+    return allow_smem(lattice_resident_kernel<T, kLat2D4, 4>, smem);
 }
 
 }  // namespace
