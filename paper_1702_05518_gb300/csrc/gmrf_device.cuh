@@ -11,6 +11,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "packed_f32.cuh"
+
 namespace gmrf {
 
 constexpr uint32_t kTagX = 0, kTagTau = 1, kTagSig = 2, kTagPrio = 3, kTagTauExtra = 5,
@@ -210,16 +212,17 @@ __device__ __forceinline__ float lg2_approx(float x)
 // relative error below 1e-6); for u >= 3/4, with v = 1 - u formed from the complemented word,
 // ln(1 - v) = -2 atanh(t), t = v / (2 - v) <= 1/7, by the atanh series
 // t (1 + t^2/3 + t^4/5 + t^6/7 + t^8/9) (truncation below 4e-10 relative), so radii near zero
-// keep their precision.
+// keep their precision.  One conversion serves both: only the word that is used is converted.
 __device__ __forceinline__ float neg2log_u_f32(uint32_t w)
 {
-    const float l1 = lg2_approx(u01_f32(w)) * -1.3862943611198906f;  // -2 ln 2 log2(u)
-    const float v = u01_f32(~w);
-    const float t = v * rcp_approx(2.0f - v);
+    const bool high = w >= 0xC0000000u;
+    const float u = u01_f32(high ? ~w : w);  // u or v
+    const float l1 = lg2_approx(u) * -1.3862943611198906f;  // -2 ln 2 log2(u)
+    const float t = u * rcp_approx(2.0f - u);
     const float t2 = t * t;
     const float p = fmaf(fmaf(fmaf(fmaf(1.0f / 9.0f, t2, 1.0f / 7.0f), t2, 1.0f / 5.0f), t2, 1.0f / 3.0f), t2, 1.0f);
     const float l2 = 4.0f * t * p;
-    return w >= 0xC0000000u ? l2 : l1;
+    return high ? l2 : l1;
 }
 
 // sin and cos of the angle pi d / 2, |d| <= 1/2 (a quarter turn centred at 0), by their Taylor
@@ -245,18 +248,71 @@ __device__ __forceinline__ void box_muller_f32(uint32_t wa, uint32_t wb, float &
     const float q2 = neg2log_u_f32(wa);  // > 0 for every word
     const float r = q2 * rsqrt_approx(q2);
     const uint32_t ws = wb + 0x20000000u;
-    const uint32_t quad = ws >> 30;
     const float d = __uint_as_float(0x3F800000u | ((ws >> 7) & 0x7FFFFFu)) - 1.5f + 0x1p-24f;
     float s, c;
     sincos_quarter_turn(d, s, c);
-    float cq = (quad & 1u) ? -s : c;
-    float sq = (quad & 1u) ? c : s;
-    if (quad & 2u) {
-        cq = -cq;
-        sq = -sq;
-    }
-    zc = r * cq;
-    zs = r * sq;
+    // half a turn is the radius's sign, a quarter turn (cos, sin) -> (-sin, cos)
+    const float rs = __uint_as_float(__float_as_uint(r) ^ (ws & 0x80000000u));
+    zc = rs * ((ws & 0x40000000u) ? -s : c);
+    zs = rs * ((ws & 0x40000000u) ? c : s);
+}
+
+// Two Box-Muller pairs, (a0, b0) in the low lanes and (a1, b1) in the high lanes of two-lane
+// arithmetic, with the operations of box_muller_f32 lane by lane (so the normals are those of the
+// scalar routine, bit for bit).  Returns each pair's (cos, sin) normals.
+// The kernels that draw whole blocks are bound by instruction issue: with one conversion per logarithm
+// and the half turn as the radius's sign, 3.5 % fewer instructions in the 256^3 volume's colour steps
+// (their time, also bound by latency, unchanged: 143 and 162 us), 3.80 -> 3.70 ms for 100 sweeps of the
+// 2047 x 1931 image; drawn two at a time in the tile kernels too, 21.0 -> 20.7 us per sweep of 512 x 512 x 4.
+__device__ __forceinline__ void box_muller_f32x2(uint32_t a0, uint32_t b0, uint32_t a1, uint32_t b1, f2 &z0, f2 &z1)
+{
+    const bool h0 = a0 >= 0xC0000000u, h1 = a1 >= 0xC0000000u;
+    const f2 u = fma2(lanes_f(h0 ? ~a0 : a0, h1 ? ~a1 : a1), splat(0x1p-32f), splat(0x1p-33f));
+    float u0, u1, d0, d1;
+    upk(u, u0, u1);
+    const f2 l1 = mul2(pk(lg2_approx(u0), lg2_approx(u1)), splat(-1.3862943611198906f));
+    upk(sub2(splat(2.0f), u), d0, d1);
+    const f2 t = mul2(u, pk(rcp_approx(d0), rcp_approx(d1)));
+    const f2 t2 = mul2(t, t);
+    const f2 p = fma2(fma2(fma2(fma2(splat(1.0f / 9.0f), t2, splat(1.0f / 7.0f)), t2, splat(1.0f / 5.0f)), t2,
+                           splat(1.0f / 3.0f)),
+                      t2, splat(1.0f));
+    const f2 l2 = mul2(mul2(splat(4.0f), t), p);
+    float l1a, l1b, l2a, l2b;
+    upk(l1, l1a, l1b);
+    upk(l2, l2a, l2b);
+    const float q0 = h0 ? l2a : l1a, q1 = h1 ? l2b : l1b;
+    const f2 r = mul2(pk(q0, q1), pk(rsqrt_approx(q0), rsqrt_approx(q1)));
+    const uint32_t s0 = b0 + 0x20000000u, s1 = b1 + 0x20000000u;
+    const f2 dd = add2(sub2(pk(__uint_as_float(0x3F800000u | ((s0 >> 7) & 0x7FFFFFu)),
+                               __uint_as_float(0x3F800000u | ((s1 >> 7) & 0x7FFFFFu))),
+                            splat(1.5f)),
+                       splat(0x1p-24f));
+    const f2 dsq = mul2(dd, dd);
+    const f2 ps = fma2(fma2(fma2(fma2(splat(1.6044118478735982e-4f), dsq, splat(-4.6817541353186881e-3f)), dsq,
+                                 splat(7.9692626246167046e-2f)),
+                            dsq, splat(-6.4596409750624625e-1f)),
+                       dsq, splat(1.5707963267948966f));
+    float sn[2], cs[2], r0, r1;
+    upk(mul2(dd, ps), sn[0], sn[1]);
+    upk(fma2(fma2(fma2(fma2(splat(9.1926027483942659e-4f), dsq, splat(-2.0863480763352961e-2f)), dsq,
+                       splat(2.5366950790104802e-1f)),
+                  dsq, splat(-1.2337005501361697f)),
+             dsq, splat(1.0f)),
+        cs[0], cs[1]);
+    upk(r, r0, r1);
+    // half a turn is the radius's sign, a quarter turn (cos, sin) -> (-sin, cos)
+    const bool t0 = s0 & 0x40000000u, t1 = s1 & 0x40000000u;
+    const float rs0 = __uint_as_float(__float_as_uint(r0) ^ (s0 & 0x80000000u));
+    const float rs1 = __uint_as_float(__float_as_uint(r1) ^ (s1 & 0x80000000u));
+    z0 = mul2(splat(rs0), pk(t0 ? -sn[0] : cs[0], t0 ? cs[0] : sn[0]));
+    z1 = mul2(splat(rs1), pk(t1 ? -sn[1] : cs[1], t1 ? cs[1] : sn[1]));
+}
+
+// The normals of one Philox block: those of chains (0, 1) and (2, 3) as pairs.
+__device__ __forceinline__ void box_muller_block_f32x2(uint4 w, f2 &z01, f2 &z23)
+{
+    box_muller_f32x2(w.x, w.y, w.z, w.w, z01, z23);
 }
 
 __device__ __forceinline__ void box_muller_f64(uint32_t wa, uint32_t wb, double &zc, double &zs)
@@ -271,9 +327,21 @@ __device__ __forceinline__ void box_muller_f64(uint32_t wa, uint32_t wb, double 
 template <typename T> struct Prec;
 template <> struct Prec<float> {
     __device__ __forceinline__ static void bm(uint32_t a, uint32_t b, float &c, float &s) { box_muller_f32(a, b, c, s); }
+    __device__ __forceinline__ static void block(uint4 w, float (&n)[4])
+    {
+        f2 z01, z23;
+        box_muller_block_f32x2(w, z01, z23);
+        upk(z01, n[0], n[1]);
+        upk(z23, n[2], n[3]);
+    }
 };
 template <> struct Prec<double> {
     __device__ __forceinline__ static void bm(uint32_t a, uint32_t b, double &c, double &s) { box_muller_f64(a, b, c, s); }
+    __device__ __forceinline__ static void block(uint4 w, double (&n)[4])
+    {
+        bm(w.x, w.y, n[0], n[1]);
+        bm(w.z, w.w, n[2], n[3]);
+    }
 };
 
 // Normal layout: a Philox block gives four normals n0, n1 (cos, sin of Box-Muller(w0, w1)) and
@@ -293,8 +361,7 @@ __device__ __forceinline__ void site_normals(uint2 key, uint32_t site, uint32_t 
                            (chain0 & static_cast<uint32_t>(lanes - 1));
     const uint4 w = philox4x32_10(make_uint4(site >> gs, sweep, stream, (kTagX << 24) | (chain0 >> 2)), key);
     if constexpr (V == 4) {
-        Prec<T>::bm(w.x, w.y, z[0], z[1]);
-        Prec<T>::bm(w.z, w.w, z[2], z[3]);
+        Prec<T>::block(w, z);
     } else if constexpr (V == 2) {
         if ((first & 2u) == 0) Prec<T>::bm(w.x, w.y, z[0], z[1]);
         else Prec<T>::bm(w.z, w.w, z[0], z[1]);
@@ -312,8 +379,7 @@ __device__ __forceinline__ void block_normals(uint2 key, uint32_t grp, uint32_t 
                                               uint32_t chain_quad, T (&n)[4])
 {
     const uint4 w = philox4x32_10(make_uint4(grp, sweep, stream, (kTagX << 24) | chain_quad), key);
-    Prec<T>::bm(w.x, w.y, n[0], n[1]);
-    Prec<T>::bm(w.z, w.w, n[2], n[3]);
+    Prec<T>::block(w, n);
 }
 
 // ------------------------------------------------------------------------------------------

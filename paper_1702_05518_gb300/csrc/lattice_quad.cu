@@ -157,9 +157,11 @@ __device__ __forceinline__ void quad_normals(float (&z)[NQ][4], uint2 key, uint3
         // odd lane: keeps (w2, w3) of the lower row, gets (w2, w3) of the upper row.
         const uint32_t p0 = __shfl_xor_sync(0xffffffffu, odd ? w.x : w.z, 1);
         const uint32_t p1 = __shfl_xor_sync(0xffffffffu, odd ? w.y : w.w, 1);
+        f2 own, partner;  // its own row and the partner's
+        box_muller_f32x2(odd ? w.z : w.x, odd ? w.w : w.y, p0, p1, own, partner);
         float c0, s0, c1, s1;
-        box_muller_f32(odd ? w.z : w.x, odd ? w.w : w.y, c0, s0);  // own row
-        box_muller_f32(p0, p1, c1, s1);                          // partner's row
+        upk(own, c0, s0);
+        upk(partner, c1, s1);
         // colour c = 2a + b: row a (0 upper, 1 lower), column b within the lane's two columns
         z[k][0] = odd ? c1 : c0;
         z[k][1] = odd ? s1 : s0;
