@@ -11,6 +11,7 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "normals_f64.cuh"
 #include "packed_f32.cuh"
 
 namespace gmrf {
@@ -263,7 +264,7 @@ __device__ __forceinline__ void box_muller_f32(uint32_t wa, uint32_t wb, float &
 // The kernels that draw whole blocks are bound by instruction issue: with one conversion per logarithm
 // and the half turn as the radius's sign, 3.5 % fewer instructions in the 256^3 volume's colour steps
 // (their time, also bound by latency, unchanged: 143 and 162 us), 3.80 -> 3.70 ms for 100 sweeps of the
-// 2047 x 1931 image; drawn two at a time in the tile kernels too, 21.0 -> 20.7 us per sweep of 512 x 512 x 4.
+// 2047 x 1931 image; drawn two at a time in the tile kernels too, 4.20 -> 4.15 ms for 300 sweeps of 512 x 512 x 3.
 __device__ __forceinline__ void box_muller_f32x2(uint32_t a0, uint32_t b0, uint32_t a1, uint32_t b1, f2 &z0, f2 &z1)
 {
     const bool h0 = a0 >= 0xC0000000u, h1 = a1 >= 0xC0000000u;
@@ -336,7 +337,7 @@ template <> struct Prec<float> {
     }
 };
 template <> struct Prec<double> {
-    __device__ __forceinline__ static void bm(uint32_t a, uint32_t b, double &c, double &s) { box_muller_f64(a, b, c, s); }
+    __device__ __forceinline__ static void bm(uint32_t a, uint32_t b, double &c, double &s) { box_muller_fixed(a, b, c, s); }
     __device__ __forceinline__ static void block(uint4 w, double (&n)[4])
     {
         bm(w.x, w.y, n[0], n[1]);
