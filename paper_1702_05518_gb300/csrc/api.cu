@@ -1597,8 +1597,8 @@ gmrf_status build_chromatic(gmrf_sampler *s, const gmrf_field_desc *fields, std:
         if (!fused_kind[s->hf[fi].kind]) total_elems += static_cast<int64_t>(s->hf[fi].n) * CV;
     const int64_t per_colour = total_elems / 2;
     // (FP64: a step is bound by the SMs' FP64 pipes, so a class of fewer elements than the SMs have
-    // threads is spread over all of them, down to 64 elements per tile: 30 x 30 x 31 sites, one chain,
-    // 42 -> 32 us per sweep; but no smaller tiles than one per SM, 48^3 with two chains 80 -> 142)
+    // threads is spread over all of them, down to 64 elements per tile; but no smaller tiles than about
+    // one per SM: 48^3 with two chains 38 us per sweep, with two and four per SM 46 and 55)
     const int64_t least = s->precision == GMRF_FP32 ? kBlock
                                                     : std::min<int64_t>(kBlock, std::max<int64_t>(64, per_colour / 140));
     const int64_t target = s->tune.step_tile ? s->tune.step_tile

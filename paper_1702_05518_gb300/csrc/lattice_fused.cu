@@ -18,6 +18,7 @@
 
 #include <type_traits>
 
+#include "fp64_steps.cuh"
 #include "gmrf_device.cuh"
 #include "gmrf_internal.h"
 #include "lattice_common.cuh"
@@ -25,20 +26,8 @@
 namespace gmrf {
 namespace {
 
-// FP64: 1/P and 1/sqrt(P) per degree and chain ([degree][Cp][2], shared memory).  P takes no other
-// values on a lattice, and two FP64 quotients and a root per site were a third of its FP64 operations.
+// FP64: 1/P and 1/sqrt(P) from a table by degree and chain (fp64_steps.cuh).
 template <typename T> constexpr bool kDegreeTable = sizeof(T) == 8;
-template <typename T>
-__device__ __forceinline__ void degree_table(T *tab, const T *hyp, int Cp, int threads)
-{
-    if constexpr (kDegreeTable<T>)
-        for (int q = threadIdx.x; q < 9 * Cp; q += threads) {
-            const int dg = q / Cp, v = q - dg * Cp;
-            const T P = hyp[v * kHypStride] * static_cast<T>(dg) + hyp[v * kHypStride + 1];
-            tab[2 * q] = FArith<T>::rcp(P);
-            tab[2 * q + 1] = FArith<T>::rsq(P);
-        }
-}
 template <typename T, int V, int KIND, int kFusedBlock>
 __global__ void __launch_bounds__(kFusedBlock, (kFusedBlock == 512 && sizeof(T) == 4 && V <= 2) ? 2 : 1)
     lattice_fused_kernel(const FusedArgs a)
@@ -86,7 +75,10 @@ __global__ void __launch_bounds__(kFusedBlock, (kFusedBlock == 512 && sizeof(T) 
         beta[v] = hyp[hc + 2];
     }
 
-    degree_table(tab, hyp + static_cast<int64_t>(t.field) * Cp * kHypStride, Cp, kFusedBlock);
+    const bool acc = a.update && a.acc_enabled && sweep_accumulated(sweep_ll, a.burn_in, a.thin);
+    __shared__ T s_inv_k;  // FP64: one quotient for the block
+    if constexpr (kDegreeTable<T>)
+        degree_table(tab, s_inv_k, hyp + static_cast<int64_t>(t.field) * Cp * kHypStride, Cp, acc, a.ctl);
 
     // Stage: rows of the NS sub-arrays; slots outside a global sub-array read as zero, and the
     // global padding slots (sites beyond an odd extent) hold zero, so every position outside
@@ -347,10 +339,10 @@ __global__ void __launch_bounds__(kFusedBlock, (kFusedBlock == 512 && sizeof(T) 
     }
 
     // Write-back of the owned sites (rows of the sub-arrays) and the running mean / M2.
-    const bool acc = a.update && a.acc_enabled && sweep_accumulated(sweep_ll, a.burn_in, a.thin);
     if (a.update) {
         T inv_k = 0;
-        if (acc) inv_k = static_cast<T>(1) / static_cast<T>(a.ctl->acc_count + 1);
+        if constexpr (kDegreeTable<T>) inv_k = s_inv_k;
+        else if (acc) inv_k = static_cast<T>(1) / static_cast<T>(a.ctl->acc_count + 1);
         T *XW = static_cast<T *>(xdst) + f.slot0 * Cp + cvo;
         T *MEAN = static_cast<T *>(a.mean) + f.slot0 * Cp + cvo;
         T *M2 = static_cast<T *>(a.m2) + f.slot0 * Cp + cvo;
@@ -569,16 +561,22 @@ __global__ void __launch_bounds__(NT, (NT == 512 && sizeof(T) == 4 && CP < 4) ? 
         }
     }
     __shared__ T tab[kDegreeTable<T> ? 9 * CP * 2 : 1];
-    degree_table(tab, static_cast<const T *>(a.hyp) + static_cast<int64_t>(t.field) * CP * kHypStride, CP, NT);
+    const bool acc = a.acc_enabled && sweep_accumulated(sweep_ll, a.burn_in, a.thin);
+    __shared__ T s_inv_k;  // FP64: one quotient for the block
+    if constexpr (kDegreeTable<T>)
+        degree_table(tab, s_inv_k, static_cast<const T *>(a.hyp) + static_cast<int64_t>(t.field) * CP * kHypStride, CP, acc,
+                     a.ctl);
     stage(X, nullptr);
     __syncthreads();
 
     // Phase B: colour steps.  An owned site is final after its own colour step: it is written
     // back then (state and, on accumulated sweeps, the running mean / M2), so the stores overlap
     // the remaining steps, and it folds its terms of the hyperparameter sums.
-    const bool acc = a.acc_enabled && sweep_accumulated(sweep_ll, a.burn_in, a.thin);
     T inv_k = 0;
-    if (acc) inv_k = static_cast<T>(1) / static_cast<T>(a.ctl->acc_count + 1);
+    if constexpr (kDegreeTable<T>) inv_k = s_inv_k;
+    else if (acc) inv_k = static_cast<T>(1) / static_cast<T>(a.ctl->acc_count + 1);
+    const bool icar = rho == static_cast<T>(1);
+    bool any_owned = false;
     T *MEAN = static_cast<T *>(a.mean) + f.slot0 * CP;
     T *M2 = static_cast<T *>(a.m2) + f.slot0 * CP;
     T accS[CP], accR[CP], accA[CP];
@@ -672,6 +670,7 @@ __global__ void __launch_bounds__(NT, (NT == 512 && sizeof(T) == 4 && CP < 4) ? 
                 }
                 T d = static_cast<T>(ND);
                 int dg = ND;
+                uint32_t miss = 0;
                 T wv[ND];
 #pragma unroll
                 for (int k = 0; k < ND; ++k) wv[k] = wl[k];
@@ -685,6 +684,7 @@ __global__ void __launch_bounds__(NT, (NT == 512 && sizeof(T) == 4 && CP < 4) ? 
                         const bool ok = ii >= 0 && ii < Hl && jj >= 0 && jj < Wl;
                         deg += ok;
                         if (!ok) wv[k] = 0;
+                        miss |= ok ? 0u : 1u << k;
                     }
                     d = static_cast<T>(deg);
                     dg = deg;
@@ -707,6 +707,7 @@ __global__ void __launch_bounds__(NT, (NT == 512 && sizeof(T) == 4 && CP < 4) ? 
                 }
                 Vec<T, CP>::st(xs + idx * CP, xn);
                 if (owned) {
+                    any_owned = true;
                     Vec<T, CP>::st(XW + go, xn);
                     if (acc) {
 #pragma unroll
@@ -724,11 +725,18 @@ __global__ void __launch_bounds__(NT, (NT == 512 && sizeof(T) == 4 && CP < 4) ? 
 #pragma unroll
                         for (int k = 0; k < ND; ++k) {
                             if (lw[k]) {  // the other directions' weights are 0: their terms add +0
-                                const T df = xn[v] - nb[k][v];
-                                e2 += wv[k] * df * df;
+                                if constexpr (kDegreeTable<T>) {
+                                    const T df = (miss >> k) & 1u ? static_cast<T>(0) : xn[v] - nb[k][v];
+                                    e2 += df * df;
+                                } else {
+                                    const T df = xn[v] - nb[k][v];
+                                    e2 += wv[k] * df * df;
+                                }
                             }
                         }
-                        accS[v] += (static_cast<T>(1) - rho) * d * xn[v] * xn[v] + rho * e2;
+                        // (FP64, rho = 1: the first term is 0 and four of a site's operations)
+                        if (kDegreeTable<T> && icar) accS[v] += e2;
+                        else accS[v] += (static_cast<T>(1) - rho) * d * xn[v] * xn[v] + rho * e2;
                         const T r = (yv - beta[v]) - xn[v];
                         accR[v] += r * r;
                         accA[v] += r;
@@ -748,19 +756,35 @@ __global__ void __launch_bounds__(NT, (NT == 512 && sizeof(T) == 4 && CP < 4) ? 
     // Block reduction (all lanes hold the same chains): warp shuffle tree, then warps in order.
     T *red = zs;  // [NW][CP][3], the normals are dead
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if constexpr (kDegreeTable<T>) {
+        const bool some = __any_sync(0xffffffffu, any_owned);  // (small tiles leave most warps without a site)
 #pragma unroll
-    for (int v = 0; v < CP; ++v) {
-        T sS = accS[v], sR = accR[v], sA = accA[v];
+        for (int v = 0; v < CP; ++v) {
+            T sSR = 0, sA = 0;
+            if (some) {
+                sSR = warp_sum_pair(accS[v], accR[v], 1);
+                sA = accA[v];
 #pragma unroll
-        for (int o = 16; o >= 1; o >>= 1) {
-            sS += __shfl_xor_sync(0xffffffffu, sS, o);
-            sR += __shfl_xor_sync(0xffffffffu, sR, o);
-            sA += __shfl_xor_sync(0xffffffffu, sA, o);
+                for (int o = 16; o >= 1; o >>= 1) sA += __shfl_xor_sync(0xffffffffu, sA, o);
+            }
+            if ((lane & 15) == 0) red[(warp * CP + v) * 3 + (lane >> 4)] = sSR;
+            if (lane == 0) red[(warp * CP + v) * 3 + 2] = sA;
         }
-        if (lane == 0) {
-            red[(warp * CP + v) * 3] = sS;
-            red[(warp * CP + v) * 3 + 1] = sR;
-            red[(warp * CP + v) * 3 + 2] = sA;
+    } else {
+#pragma unroll
+        for (int v = 0; v < CP; ++v) {
+            T sS = accS[v], sR = accR[v], sA = accA[v];
+#pragma unroll
+            for (int o = 16; o >= 1; o >>= 1) {
+                sS += __shfl_xor_sync(0xffffffffu, sS, o);
+                sR += __shfl_xor_sync(0xffffffffu, sR, o);
+                sA += __shfl_xor_sync(0xffffffffu, sA, o);
+            }
+            if (lane == 0) {
+                red[(warp * CP + v) * 3] = sS;
+                red[(warp * CP + v) * 3 + 1] = sR;
+                red[(warp * CP + v) * 3 + 2] = sA;
+            }
         }
     }
     __syncthreads();

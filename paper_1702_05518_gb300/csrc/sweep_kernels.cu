@@ -22,6 +22,7 @@
 
 #include <type_traits>
 
+#include "fp64_steps.cuh"
 #include "gmrf_device.cuh"
 #include "gmrf_internal.h"
 #include "gamma_pre.cuh"
@@ -53,10 +54,8 @@ struct SiteCtx {
     T accS[V], accR[V], accA[V]; // thread partial sums
     T inv_k;             // 1 / (accumulated count) when accumulating
     bool acc;
-    // FP64 lattices: 1/P and 1/sqrt(P) per degree and chain ([degree][Cp][2], shared memory).  P takes
-    // no other values without weights, and the two FP64 quotients and the root were a third of a site's
-    // FP64 operations.
-    const T *tab;
+    const T *tab;        // FP64 lattices: 1/P and 1/sqrt(P) by degree and chain (fp64_steps.cuh)
+    bool icar;           // rho = 1
 };
 // Whether a kernel uses that table.
 template <typename T, int KIND, int MODEL> constexpr bool kDegreeTable = sizeof(T) == 8 && KIND != kCsr && MODEL != kModelBinomial;
@@ -74,7 +73,8 @@ template <typename T, int V, int NB, int MODEL, bool TAB = false>
 __device__ __forceinline__ void finish_site(const StepArgs &a, SiteCtx<T, V> &cx, T *xp, T *meanp, T *m2p,
                                             T yv, int mtr, T d, uint32_t site, uint32_t sweep, uint32_t stream,
                                             uint32_t chain0, const T (&s)[V], const T (&nb)[NB][V],
-                                            uint32_t lower_mask, const T (&wnb)[NB], const T *zdrawn = nullptr)
+                                            uint32_t lower_mask, const T (&wnb)[NB], const T *zdrawn = nullptr,
+                                            int dg = 0)
 {
     const T rho = static_cast<T>(a.rho);
     T xn[V];
@@ -116,7 +116,7 @@ __device__ __forceinline__ void finish_site(const StepArgs &a, SiteCtx<T, V> &cx
 #pragma unroll
         for (int v = 0; v < V; ++v) {
             if constexpr (TAB) {
-                const T *q = cx.tab + (static_cast<int>(d) * a.Cp + static_cast<int>(chain0) + v) * 2;
+                const T *q = cx.tab + (dg * a.Cp + static_cast<int>(chain0) + v) * 2;
                 const T m = (cx.tau[v] * rho * s[v] + (yv - cx.beta[v]) * cx.isig[v]) * q[0];
                 xn[v] = m + z[v] * q[1];
             } else {
@@ -141,7 +141,9 @@ __device__ __forceinline__ void finish_site(const StepArgs &a, SiteCtx<T, V> &cx
                 e += wnb[k] * df * df;
             }
         }
-        cx.accS[v] += (static_cast<T>(1) - rho) * d * xn[v] * xn[v] + rho * e;
+        // (FP64 lattices, rho = 1: the first term is 0 and four of a site's operations)
+        if (TAB && cx.icar) cx.accS[v] += e;
+        else cx.accS[v] += (static_cast<T>(1) - rho) * (TAB ? static_cast<T>(dg) : d) * xn[v] * xn[v] + rho * e;
         if (MODEL == kModelBinomial) {
             cx.accR[v] += psi[v];
             cx.accA[v] += kappa - psi[v] * xn[v];
@@ -240,7 +242,8 @@ __device__ void lattice_parity_tile(const StepArgs &a, const FieldDev &f, const 
         const uint32_t site = static_cast<uint32_t>(r * W + j);
         const int mtr = MODEL == kModelBinomial ? a.trials[self_base + rb] : 0;
         finish_site<T, V, NB, MODEL, kDegreeTable<T, kLat3D6, MODEL>>(a, cx, XS + rb * Cp, MS + rb * Cp, QS + rb * Cp, YS[rb], mtr, static_cast<T>(__popc(valid)),
-                              site, sweep, f.stream, static_cast<uint32_t>(cv * V), s, nb, lower_all & valid, wnb);
+                              site, sweep, f.stream, static_cast<uint32_t>(cv * V), s, nb, lower_all & valid, wnb, nullptr,
+                              __popc(valid));
     }
 }
 
@@ -320,7 +323,7 @@ __device__ void lattice8_tile(const StepArgs &a, const FieldDev &f, const Tile &
         const int mtr = MODEL == kModelBinomial ? a.trials[f.slot0 + static_cast<int64_t>(c) * sub + base] : 0;
         finish_site<T, V, NB, MODEL, kDegreeTable<T, kLat2D8, MODEL>>(a, cx, XS + base * Cp, MS + base * Cp, QS + base * Cp, YS[base], mtr,
                               static_cast<T>(__popc(valid)), site, sweep, f.stream, static_cast<uint32_t>(cv * V),
-                              s, nb, lower & valid, wnb);
+                              s, nb, lower & valid, wnb, nullptr, __popc(valid));
     }
 }
 
@@ -453,8 +456,10 @@ __device__ void csr_tile(const StepArgs &a, const FieldDev &f, const Tile &t, Si
 
 // MODEL: the observation model; without the intercept beta0 = 0 and the third sum is not
 // needed, which the compiler then removes, registers included.
+// FP64: two blocks per SM (128 registers), or a class of more tiles than SMs runs in two waves (48^3, two chains,
+// 231 tiles: 44 us per sweep against 38).
 template <typename T, int V, int KIND, int MODEL>
-__global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? (KIND == kCsr ? 2 : 3) : 1) colour_step_kernel(const StepArgs a)
+__global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? (KIND == kCsr ? 2 : 3) : 2) colour_step_kernel(const StepArgs a)
 {
     // Tiles and fields are never written by a sweep: read before the dependency wait.
     const Tile t = a.tiles[blockIdx.x];
@@ -481,22 +486,19 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? (KIND == kCsr ? 2 : 3
     }
     cx.acc = false;
     cx.inv_k = 0;
+    constexpr bool kTab = kDegreeTable<T, KIND, MODEL>;
     if (a.update && a.acc_enabled && sweep_accumulated(sweep_ll, a.burn_in, a.thin)) {
         cx.acc = true;
-        cx.inv_k = static_cast<T>(1) / static_cast<T>(a.ctl->acc_count + 1);
+        if (!kTab) cx.inv_k = static_cast<T>(1) / static_cast<T>(a.ctl->acc_count + 1);
     }
 
-    __shared__ T tab[kDegreeTable<T, KIND, MODEL> ? 9 * kMaxChains * 2 : 1];
+    __shared__ T tab[kTab ? 9 * kMaxChains * 2 : 1], s_inv_k;
     cx.tab = tab;
-    if constexpr (kDegreeTable<T, KIND, MODEL>) {
-        for (int q = threadIdx.x; q < 9 * a.Cp; q += kBlock) {
-            const int dg = q / a.Cp, v = q - dg * a.Cp;
-            const T *hv = hyp + (static_cast<int64_t>(t.field) * a.Cp + v) * kHypStride;
-            const T P = hv[0] * static_cast<T>(dg) + hv[1];
-            tab[2 * q] = Arith<T>::rcp(P);
-            tab[2 * q + 1] = Arith<T>::rsq(P);
-        }
+    cx.icar = a.rho == 1.0;
+    if constexpr (kTab) {
+        degree_table(tab, s_inv_k, hyp + static_cast<int64_t>(t.field) * a.Cp * kHypStride, a.Cp, cx.acc, a.ctl);
         __syncthreads();
+        cx.inv_k = s_inv_k;
     }
 
     const int cv_shift = __ffs(CV) - 1;
@@ -515,10 +517,18 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? (KIND == kCsr ? 2 : 3
         T sS = cx.accS[v];
         T sR = cx.accR[v];
         T sA = MODEL != kModelGauss ? cx.accA[v] : static_cast<T>(0);
-        for (int off = 16; off >= CV; off >>= 1) {
-            sS += __shfl_xor_sync(0xffffffffu, sS, off);
-            sR += __shfl_xor_sync(0xffffffffu, sR, off);
-            if (MODEL != kModelGauss) sA += __shfl_xor_sync(0xffffffffu, sA, off);
+        if constexpr (kTab) {
+            if (CV <= 16) {
+                sS = warp_sum_pair(sS, sR, CV);
+                sR = __shfl_xor_sync(0xffffffffu, sS, 16);
+            }
+            for (int off = 16; off >= CV && MODEL != kModelGauss; off >>= 1) sA += __shfl_xor_sync(0xffffffffu, sA, off);
+        } else {
+            for (int off = 16; off >= CV; off >>= 1) {
+                sS += __shfl_xor_sync(0xffffffffu, sS, off);
+                sR += __shfl_xor_sync(0xffffffffu, sR, off);
+                if (MODEL != kModelGauss) sA += __shfl_xor_sync(0xffffffffu, sA, off);
+            }
         }
         if (lane < CV) {
             red[warp][lane * V + v][0] = sS;

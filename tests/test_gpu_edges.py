@@ -69,6 +69,24 @@ def test_fp64_tiles_and_degrees(kind, dims, chains):
             assert trace_relerr(r["tau_trace"], out["tau_trace"][c]) <= TOL_FP64
 
 
+@pytest.mark.parametrize("chains", [20, 40])  # 16 and 32 chain vectors to a warp
+@pytest.mark.parametrize("rho", [1.0, 0.7])
+@pytest.mark.parametrize("kind,dims,flags", [(wl.LATTICE3D_6, (3, 4, 5), 0), (wl.LATTICE2D_8, (9, 7), g.FLAG_PER_COLOUR),
+                                             (wl.LATTICE2D_4, (9, 7), 0)])
+def test_fp64_sums_of_many_chains(kind, dims, flags, chains, rho):
+    f = wl.small_lattice(kind, dims, 16)
+    st, out = run_oracle(f, chains, 4, seed=8, stream=0, prior="icar" if rho == 1.0 else "pcar", rho=rho, burn_in=1,
+                         intercept=True)
+    with g.Sampler([f], precision=g.FP64, chains=chains, seed=8, prior=g.PRIOR_ICAR if rho == 1.0 else g.PRIOR_PCAR,
+                   rho=rho, burn_in=1, intercept=True, flags=flags) as s:
+        s.sweep(4)
+        for c in (0, 1, chains - 1):
+            r = s.fetch(0, c, trace=4)
+            assert relerr(r["x"], st.x[c]) <= TOL_FP64 and relerr(r["mean"], st.mean[c]) <= TOL_FP64
+            assert trace_relerr(r["tau_trace"], out["tau_trace"][c]) <= TOL_FP64
+            assert trace_relerr(r["sigma2_trace"], out["sigma2_trace"][c]) <= TOL_FP64
+
+
 @pytest.mark.parametrize("precision", [g.FP32, g.FP64])
 @pytest.mark.parametrize("chains", [1, 2, 3, 5, 8, 11, 16])
 def test_pooled_moments(precision, chains):
