@@ -731,7 +731,7 @@ cudaError_t plan_tile_resident(gmrf_sampler *s)
                                                       &fits);
     if (e != cudaSuccess || !fits) return e;
     if (s->Cp == 4) {
-        const cudaError_t ea = s->alloc_t(&s->res_pm, static_cast<size_t>(3) * s->Cp * s->ftile_cnt[kind], sizeof(double));
+        const cudaError_t ea = s->alloc_t(&s->res_pm, static_cast<size_t>(2) * 3 * s->Cp * s->ftile_cnt[kind], sizeof(double));
         if (ea != cudaSuccess) return ea;
     }
     s->res_batch = std::min(128, std::max(64, s->opts.graph_sweeps));
@@ -1772,7 +1772,8 @@ gmrf_status build_chromatic(gmrf_sampler *s, const gmrf_field_desc *fields, std:
     if (!fall.empty())
         CK(cudaMemcpyAsync(s->ftiles_dev, fall.data(), sizeof(TileXY) * fall.size(), cudaMemcpyHostToDevice,
                            s->stream));
-    CK(s->alloc_t(&s->partials, static_cast<size_t>(std::max(part, 1)) * Cp, sizeof(Part3)));
+    // (a second set for the tile kernels that keep a single field resident, by the sweep's parity)
+    CK(s->alloc_t(&s->partials, static_cast<size_t>(std::max(part, 1)) * (s->nfields == 1 ? 2 : 1) * Cp, sizeof(Part3)));
     CK(cudaMemsetAsync(s->partials, 0, static_cast<size_t>(std::max(part, 1)) * Cp * sizeof(Part3), s->stream));
     CK(cudaMemcpyAsync(s->fields_dev, s->fd.data(), sizeof(FieldDev) * s->nfields, cudaMemcpyHostToDevice, s->stream));
 

@@ -384,8 +384,11 @@ __global__ void __launch_bounds__(NT, (NT == 512 && CP < 4) ? 2 : 1) lattice_fus
             const int chain = tid / 3, k = tid - 3 * chain;
             T sum = 0;
             for (int w = 0; w < NW; ++w) sum += red[(w * CP + chain) * 3 + k];
-            reinterpret_cast<double *>(a.partials + static_cast<int64_t>(t.part) * CP + chain)[k] = static_cast<double>(sum);
-            if (CP == 4) ra.pm[(chain * 3 + k) * f.nparts + (t.part - f.part0)] = static_cast<double>(sum);
+            // by the sweep's parity: a tile cut short by the lattice's edge ends its next sweep while others may
+            // still be drawing ahead, before they read this one's sums
+            const int part = t.part + (it & 1) * f.nparts;
+            reinterpret_cast<double *>(a.partials + static_cast<int64_t>(part) * CP + chain)[k] = static_cast<double>(sum);
+            if (CP == 4) ra.pm[((it & 1) * CP * 3 + chain * 3 + k) * f.nparts + (t.part - f.part0)] = static_cast<double>(sum);
         }
         __syncthreads();  // the partial and every owned site of the sweep are stored; `red` is free
 
@@ -434,12 +437,12 @@ __global__ void __launch_bounds__(NT, (NT == 512 && CP < 4) ? 2 : 1) lattice_fus
                 // sweep of the 512 x 512 image with the intercept; with one or two chains the
                 // records' reads measured faster)
                 if (CP == 4) {
-                    const double *pc = ra.pm + chain * 3 * f.nparts;
+                    const double *pc = ra.pm + ((it & 1) * CP + chain) * 3 * f.nparts;
                     hyper_sums_by_field(pc + which * f.nparts, pc + 2 * f.nparts, need_a, f.nparts, S, A);
                 } else if (h.max_parts >= 256) {
-                    hyper_sums<true, true>(h, which, need_a, chain, f.part0, f.nparts, S, A);
+                    hyper_sums<true, true>(h, which, need_a, chain, f.part0 + (it & 1) * f.nparts, f.nparts, S, A);
                 } else {
-                    hyper_sums<false, true>(h, which, need_a, chain, f.part0, f.nparts, S, A);
+                    hyper_sums<false, true>(h, which, need_a, chain, f.part0 + (it & 1) * f.nparts, f.nparts, S, A);
                 }
             }
             if (lane == 0) {

@@ -502,7 +502,9 @@ __global__ void __launch_bounds__(NT, 1) lattice_quad_resident_kernel(const Tile
         if (tid < 3) {
             float sum = 0.0f;
             for (int w = 0; w < NW; ++w) sum += red[w][tid];
-            reinterpret_cast<double *>(a.partials + t.part)[tid] = static_cast<double>(sum);
+            // by the sweep's parity: a tile cut short by the lattice's edge ends its next sweep while others may
+            // still be drawing ahead, before they read this one's sums
+            reinterpret_cast<double *>(a.partials + t.part + (it & 1) * f.nparts)[tid] = static_cast<double>(sum);
         }
         __syncthreads();  // the partial and every owned site of the sweep are stored
 
@@ -555,7 +557,7 @@ __global__ void __launch_bounds__(NT, 1) lattice_quad_resident_kernel(const Tile
             const bool need_sum = which ? (h.draw || h.draw_beta) : h.draw;
             const bool need_a = which && h.draw_beta;
             double S = 0.0, A = 0.0;
-            if (need_sum) hyper_sums<false, true>(h, which, need_a, 0, f.part0, f.nparts, S, A);
+            if (need_sum) hyper_sums<false, true>(h, which, need_a, 0, f.part0 + (it & 1) * f.nparts, f.nparts, S, A);
             if (lane == 0) {
                 const long long kb = sw - bbase;
                 const bool pre = h.gpre && kb >= 0 && kb < bcount;
