@@ -190,9 +190,12 @@ typedef struct {
  * every thread holds all chains (1, 2 or 4 in the layout).  An FP32 sampler of up to 8
  * chains of a single graph beyond the small ones (weighted edges, more sites, neighbours or sites per
  * class) or of a single 3-D lattice of up to about 1.2 million sites (one chain; 0.6 million with two,
- * 0.3 million with four, 0.15 million with eight) runs its colour steps in one cooperative launch per batch of sweeps as well, with a grid barrier
- * per colour step (results equal up to rounding; its state stays in device memory, and
- * gmrf_info.resident stays 0), unless a tuning of the colour-step kernels is given.  On by default in FP32;
+ * 0.3 million with four, 0.15 million with eight) runs its colour steps in one cooperative launch per
+ * batch of sweeps as well, with a grid barrier per colour step (results equal up to rounding; its
+ * state stays in device memory, and gmrf_info.resident stays 0), unless a tuning of the colour-step
+ * kernels is given.  So does an FP32 sampler of one or two chains of a single 2-D lattice whose tiles do
+ * not fit in one wave: marching warps, a grid barrier per sweep (gmrf_info.resident 0; unless a tuning of
+ * the tiled kernels is given).  On by default in FP32;
  * GMRF_FLAG_RESIDENT asks for the small-lattice form in FP64 as well, GMRF_FLAG_NO_RESIDENT keeps
  * the per-sweep launches.
  * gmrf_info.resident tells which path a sampler took. */

@@ -12,21 +12,21 @@
 // Vertical neighbours are the lane's own registers and horizontal ones a warp shuffle away: no shared
 // memory and no block barrier in a sweep.  The sites beyond the strip and chunk that its own sites
 // depend on are drawn again (identically: the draws are functions of their counters): one lane on
-// either side (two columns would do for the 4-neighbour lattice, four for the other), and a row above
-// and below (an even row below).  The new state goes to the other of two buffers, so no warp reads a
+// either side (two for the 8-neighbour lattice with two chains: it needs four columns, the other two), and a
+// row above and below (an even row below).  The new state goes to the other of two buffers, so no warp reads a
 // neighbour's new values, and each owned site's terms of the two sums of the conjugate draws and its
 // running moments are folded in as it is drawn.
 //
-// One Philox block serves the NC sites of a lane and row (one chain), two of them (two chains) or one
-// (more); where a row starts within a block (one or two chains and a row length that is no multiple),
-// the normals move over by that offset through a shuffle.
+// A lane has four columns with one chain and two with two, one Philox block's normals for its sites of a
+// row; where a row starts within a block (a row length that is no multiple), the normals move over by
+// that offset through a shuffle.
 //
 // Two forms of the same arithmetic in the same order, block for block: one launch per sweep (samplers
 // of several fields, or without the resident path), and a batch of sweeps of a single field in one
 // cooperative launch (a grid barrier per sweep, every block drawing the parameters; the normals of a
 // chunk's first rows are drawn into shared memory while the barrier completes).
 //
-// Bound by instruction issue: about 105 instructions per site-update, 35 of them the normals (the
+// Bound by instruction issue: about 103 instructions per site-update, 33 of them the normals (the
 // tiled kernel of lattice_fused.cu, whose threads walk shared-memory tiles colour by colour, takes 300
 // to 340).  Per sweep, against that kernel and a launch for the draws: 4-neighbour 2047 x 1931 one
 // chain 24 us (46 without accumulation, 58 with, and 8), 8-neighbour 2048 x 2048 one chain 26 (49,
