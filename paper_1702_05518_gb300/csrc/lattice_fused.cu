@@ -26,7 +26,7 @@
 namespace gmrf {
 namespace {
 
-// FP64: 1/P and 1/sqrt(P) from a table by degree and chain (fp64_steps.cuh).
+// FP64: the draws' coefficients from a table by degree and chain (fp64_steps.cuh).
 template <typename T> constexpr bool kDegreeTable = sizeof(T) == 8;
 template <typename T, int V, int KIND, int kFusedBlock>
 __global__ void __launch_bounds__(kFusedBlock, (kFusedBlock == 512 && sizeof(T) == 4 && V <= 2) ? 2 : 1)
@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(kFusedBlock, (kFusedBlock == 512 && sizeof(T) 
     const uint32_t sweep = static_cast<uint32_t>(sweep_ll);
     const T rho = static_cast<T>(a.rho);
 
-    __shared__ T tab[kDegreeTable<T> ? 9 * kMaxChains * 2 : 1];
+    __shared__ T tab[kDegreeTable<T> ? 9 * kMaxChains * 3 : 1];
     T tau[V], isig[V], beta[V];
     const T *hyp = static_cast<const T *>(a.hyp);
 #pragma unroll
@@ -78,7 +78,7 @@ __global__ void __launch_bounds__(kFusedBlock, (kFusedBlock == 512 && sizeof(T) 
     const bool acc = a.update && a.acc_enabled && sweep_accumulated(sweep_ll, a.burn_in, a.thin);
     __shared__ T s_inv_k;  // FP64: one quotient for the block
     if constexpr (kDegreeTable<T>)
-        degree_table(tab, s_inv_k, hyp + static_cast<int64_t>(t.field) * Cp * kHypStride, Cp, acc, a.ctl);
+        degree_table(tab, s_inv_k, hyp + static_cast<int64_t>(t.field) * Cp * kHypStride, Cp, a.rho, acc, a.ctl);
 
     // Stage: rows of the NS sub-arrays; slots outside a global sub-array read as zero, and the
     // global padding slots (sites beyond an odd extent) hold zero, so every position outside
@@ -270,9 +270,7 @@ __global__ void __launch_bounds__(kFusedBlock, (kFusedBlock == 512 && sizeof(T) 
 #pragma unroll
             for (int v = 0; v < V; ++v) {
                 if constexpr (kDegreeTable<T>) {
-                    const T *q = tab + (deg * Cp + cvo + v) * 2;
-                    const T m = (tau[v] * rho * s[v] + (yv - beta[v]) * isig[v]) * q[0];
-                    xn[v] = m + z[v] * q[1];
+                    xn[v] = table_draw(tab + (deg * Cp + cvo + v) * 3, pair_sum<D::N>(&nb[0][v], V), yv - beta[v], z[v]);
                 } else {
                     const T P = tau[v] * d + isig[v];
                     const T m = (tau[v] * rho * s[v] + (yv - beta[v]) * isig[v]) * FArith<T>::rcp(P);
@@ -406,7 +404,9 @@ __global__ void __launch_bounds__(kFusedBlock, (kFusedBlock == 512 && sizeof(T) 
     for (int q = threadIdx.x; q < Cp * 3; q += kFusedBlock) {
         const int chain = q / 3, k = q - 3 * chain;
         T sum = 0;
-        for (int w = 0; w < NW; ++w) sum += red[(w * Cp + chain) * 3 + k];
+        if constexpr (kDegreeTable<T>) sum = pair_sum<NW>(red + chain * 3 + k, Cp * 3);
+        else
+            for (int w = 0; w < NW; ++w) sum += red[(w * Cp + chain) * 3 + k];
         reinterpret_cast<double *>(a.partials + static_cast<int64_t>(t.part) * Cp + chain)[k] = static_cast<double>(sum);
     }
 }
@@ -560,12 +560,12 @@ __global__ void __launch_bounds__(NT, (NT == 512 && sizeof(T) == 4 && CP < 4) ? 
             beta[v] = hyp[kHypStride * v + 2];
         }
     }
-    __shared__ T tab[kDegreeTable<T> ? 9 * CP * 2 : 1];
+    __shared__ T tab[kDegreeTable<T> ? 9 * CP * 3 : 1];
     const bool acc = a.acc_enabled && sweep_accumulated(sweep_ll, a.burn_in, a.thin);
     __shared__ T s_inv_k;  // FP64: one quotient for the block
     if constexpr (kDegreeTable<T>)
-        degree_table(tab, s_inv_k, static_cast<const T *>(a.hyp) + static_cast<int64_t>(t.field) * CP * kHypStride, CP, acc,
-                     a.ctl);
+        degree_table(tab, s_inv_k, static_cast<const T *>(a.hyp) + static_cast<int64_t>(t.field) * CP * kHypStride, CP, a.rho,
+                     acc, a.ctl);
     stage(X, nullptr);
     __syncthreads();
 
@@ -696,9 +696,7 @@ __global__ void __launch_bounds__(NT, (NT == 512 && sizeof(T) == 4 && CP < 4) ? 
 #pragma unroll
                 for (int v = 0; v < CP; ++v) {
                     if constexpr (kDegreeTable<T>) {
-                        const T *q = tab + (dg * CP + v) * 2;
-                        const T m = (tau[v] * rho * s[v] + (yv - beta[v]) * isig[v]) * q[0];
-                        xn[v] = m + z[v] * q[1];
+                        xn[v] = table_draw(tab + (dg * CP + v) * 3, pair_sum<ND>(&nb[0][v], CP), yv - beta[v], z[v]);
                     } else {
                         const T P = tau[v] * d + isig[v];
                         const T m = (tau[v] * rho * s[v] + (yv - beta[v]) * isig[v]) * FArith<T>::rcp(P);
@@ -791,7 +789,9 @@ __global__ void __launch_bounds__(NT, (NT == 512 && sizeof(T) == 4 && CP < 4) ? 
     if (threadIdx.x < CP * 3) {
         const int chain = threadIdx.x / 3, k = threadIdx.x - 3 * chain;
         T sum = 0;
-        for (int w = 0; w < NW; ++w) sum += red[(w * CP + chain) * 3 + k];
+        if constexpr (kDegreeTable<T>) sum = pair_sum<NW>(red + chain * 3 + k, CP * 3);
+        else
+            for (int w = 0; w < NW; ++w) sum += red[(w * CP + chain) * 3 + k];
         reinterpret_cast<double *>(a.partials + static_cast<int64_t>(t.part) * CP + chain)[k] = static_cast<double>(sum);
     }
 }

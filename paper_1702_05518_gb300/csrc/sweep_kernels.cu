@@ -54,7 +54,7 @@ struct SiteCtx {
     T accS[V], accR[V], accA[V]; // thread partial sums
     T inv_k;             // 1 / (accumulated count) when accumulating
     bool acc;
-    const T *tab;        // FP64 lattices: 1/P and 1/sqrt(P) by degree and chain (fp64_steps.cuh)
+    const T *tab;        // FP64 lattices: the draws' coefficients by degree and chain (fp64_steps.cuh)
     bool icar;           // rho = 1
 };
 // Whether a kernel uses that table.
@@ -116,9 +116,8 @@ __device__ __forceinline__ void finish_site(const StepArgs &a, SiteCtx<T, V> &cx
 #pragma unroll
         for (int v = 0; v < V; ++v) {
             if constexpr (TAB) {
-                const T *q = cx.tab + (dg * a.Cp + static_cast<int>(chain0) + v) * 2;
-                const T m = (cx.tau[v] * rho * s[v] + (yv - cx.beta[v]) * cx.isig[v]) * q[0];
-                xn[v] = m + z[v] * q[1];
+                xn[v] = table_draw(cx.tab + (dg * a.Cp + static_cast<int>(chain0) + v) * 3, pair_sum<NB>(&nb[0][v], V),
+                                   yv - cx.beta[v], z[v]);
             } else {
                 const T P = cx.tau[v] * d + cx.isig[v];
                 const T m = (cx.tau[v] * rho * s[v] + (yv - cx.beta[v]) * cx.isig[v]) * Arith<T>::rcp(P);
@@ -492,11 +491,11 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? (KIND == kCsr ? 2 : 3
         if (!kTab) cx.inv_k = static_cast<T>(1) / static_cast<T>(a.ctl->acc_count + 1);
     }
 
-    __shared__ T tab[kTab ? 9 * kMaxChains * 2 : 1], s_inv_k;
+    __shared__ T tab[kTab ? 9 * kMaxChains * 3 : 1], s_inv_k;
     cx.tab = tab;
     cx.icar = a.rho == 1.0;
     if constexpr (kTab) {
-        degree_table(tab, s_inv_k, hyp + static_cast<int64_t>(t.field) * a.Cp * kHypStride, a.Cp, cx.acc, a.ctl);
+        degree_table(tab, s_inv_k, hyp + static_cast<int64_t>(t.field) * a.Cp * kHypStride, a.Cp, a.rho, cx.acc, a.ctl);
         __syncthreads();
         cx.inv_k = s_inv_k;
     }
@@ -540,7 +539,9 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? (KIND == kCsr ? 2 : 3
     for (int q = threadIdx.x; q < a.Cp * 3; q += kBlock) {
         const int chain = q / 3, k = q - 3 * chain;
         T acc = 0;
-        for (int w = 0; w < kBlock / 32; ++w) acc += red[w][chain][k];
+        if constexpr (kTab) acc = pair_sum<kBlock / 32>(&red[0][chain][k], kMaxChains * 3);
+        else
+            for (int w = 0; w < kBlock / 32; ++w) acc += red[w][chain][k];
         double *dst = reinterpret_cast<double *>(a.partials + static_cast<int64_t>(t.part) * a.Cp + chain);
         dst[k] = static_cast<double>(acc);
     }

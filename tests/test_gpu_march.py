@@ -121,3 +121,19 @@ def test_sums_of_an_extra_draw(kind, chains):
             s.hyper_update()
             out.append([(s.fetch(0, c)["tau"], s.fetch(0, c)["sigma2"]) for c in range(chains)])
     assert np.allclose(out[0], out[1], rtol=1e-5, atol=0)
+
+
+def test_barrier_timeout_reports_and_poisons():
+    f = wl.small_lattice(wl.LATTICE2D_4, (41, 241), 13)
+    with g.Sampler([f], precision=g.FP32, chains=1, seed=3, flags=g.FLAG_TEST_STALL, **_march(1)) as s:
+        assert s.info()["resident"] == 0
+        s.sweep(10)
+        with pytest.raises(g.GmrfError) as e:
+            s.fetch(0, 0)
+        assert e.value.status == g.E_TIMEOUT
+        with pytest.raises(g.GmrfError) as e:
+            s.sweep(1)
+        assert e.value.status == g.E_STATE
+    res, info = _run([f], 1, [10], **_march(1))
+    assert info["wait_timeouts"] == 0
+    _check(f, res[0], 1, 10, TOL_FP32_1000)
