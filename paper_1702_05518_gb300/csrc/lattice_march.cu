@@ -26,7 +26,8 @@
 // cooperative launch (a grid barrier per sweep, every block drawing the parameters; the normals of a
 // chunk's first rows are drawn into shared memory while the barrier completes).
 //
-// Bound by instruction issue: about 103 instructions per site-update, 33 of them the normals (the
+// Bound by instruction issue and its latencies (126 registers: four warps per scheduler, 47 % issue): about
+// 124 instructions per site-update, 33 of them the normals and a fifth for sites drawn again (the
 // tiled kernel of lattice_fused.cu, whose threads walk shared-memory tiles colour by colour, takes 300
 // to 340).  Per sweep, against that kernel and a launch for the draws: 4-neighbour 2047 x 1931 one
 // chain 24 us (46 without accumulation, 58 with, and 8), 8-neighbour 2048 x 2048 one chain 26 (49,
