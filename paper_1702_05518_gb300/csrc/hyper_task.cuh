@@ -32,12 +32,14 @@ namespace gmrf {
 // sweep used, gpv and zb the precomputed Gamma variate and normal when `pre`.  With `rec`, writes
 // the FP64 values, the precision-T copies and the traces (without it the caller only takes the
 // results: the blocks of the resident quad kernel that draw redundantly); returns the parameter's
-// new value (tau or sigma^2) in val and, for task 1, beta0 in bval.
+// new value (tau or sigma^2) in val and, for task 1, beta0 in bval.  `root`: sqrt(s2old / n), where the
+// caller has computed it while it waited.
 template <typename T>
 __device__ __forceinline__ void hyper_draw(const HyperArgs &a, int which, int chain, int64_t hc, long long sweep,
                                            double S, double A, double cur, double s2old, double b, double gpv,
                                            double zb, bool pre, long long extra, uint32_t fstream, int32_t fn,
-                                           int32_t frank, double &val_out, double &bval_out, bool rec = true)
+                                           int32_t frank, double &val_out, double &bval_out, bool rec = true,
+                                           const double *root = nullptr)
 {
     T *hyp = static_cast<T *>(a.hyp);
     const uint32_t word1 = static_cast<uint32_t>(a.end_of_sweep ? sweep : extra);
@@ -56,7 +58,7 @@ __device__ __forceinline__ void hyper_draw(const HyperArgs &a, int which, int ch
             const double Pb = 1.0 / a.beta0_var + S;
             bval = (a.beta0_mean / a.beta0_var + A) / Pb + zb / sqrt(Pb);
         } else {
-            const double delta = A / fn + sqrt(s2old / fn) * zb;
+            const double delta = A / fn + (root ? *root : sqrt(s2old / fn)) * zb;
             bval = b + delta;
             S = S - 2.0 * delta * A + fn * (delta * delta);
         }

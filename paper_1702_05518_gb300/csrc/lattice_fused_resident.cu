@@ -57,7 +57,10 @@ template <> struct LdCg<4> {
     }
 };
 
-template <int KIND, int NT, int CP>
+// ICPT: the launch draws beta0.  The scale of that draw, sqrt(sigma^2 / n), needs no sum of the sweep: 0.7 us of
+// dependent FP64 operations that then run beside the normals (512 x 512, three chains, 300 sweeps: 4.15 ->
+// 4.00 ms; decided at run time, it cost the launches without the intercept 0.4 %).
+template <int KIND, int NT, int CP, bool ICPT>
 __global__ void __launch_bounds__(NT, (NT == 512 && CP < 4) ? 2 : 1) lattice_fused_resident(const TileResArgs ra)
 {
     using T = float;
@@ -71,6 +74,11 @@ __global__ void __launch_bounds__(NT, (NT == 512 && CP < 4) ? 2 : 1) lattice_fus
     const HyperArgs &h = ra.h;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ T hs[CP][3];          // tau, 1/sigma^2, beta0 of the current sweep per chain
+    double *root = nullptr;  // sqrt(sigma^2 / n)
+    if constexpr (ICPT) {
+        __shared__ double s_root[CP];
+        root = s_root;
+    }
     __shared__ double dcur[CP][2];   // tau and sigma^2 (FP64) as last drawn, per chain
     __shared__ double gsh[kResGpre][CP][3];
     __shared__ int s_abort;
@@ -394,6 +402,8 @@ __global__ void __launch_bounds__(NT, (NT == 512 && CP < 4) ? 2 : 1) lattice_fus
 
         // Grid barrier: arrive, draw the next sweep's normals, then wait (bounded).
         if (tid == 0) grid_arrive(ctl);
+        // (by the last warps, which have the fewest normals)
+        if (ICPT && NW - 1 - warp < CP && lane == 0) root[NW - 1 - warp] = sqrt(dcur[NW - 1 - warp][1] / f.n);
         if (it + 1 < ra.count) normals(static_cast<uint32_t>(sw + 1));
         if (tid == 0) {
             const unsigned long long target = (static_cast<unsigned long long>(it) + 1) * nblk + ra.extra_arrivals;
@@ -464,7 +474,7 @@ __global__ void __launch_bounds__(NT, (NT == 512 && CP < 4) ? 2 : 1) lattice_fus
                 const double b = which ? static_cast<double>(hs[chain][2]) : 0.0;
                 double val, bval;
                 hyper_draw<float>(h, which, chain, chain, sw, S, A, cur, s2old, b, gpv, zb, pre, 0, f.stream, f.n,
-                                  f.rank, val, bval, blockIdx.x == 0);
+                                  f.rank, val, bval, blockIdx.x == 0, ICPT ? &root[chain] : nullptr);
                 if (which == 0) {
                     if (h.draw) hs[chain][0] = static_cast<T>(val);
                 } else {
@@ -508,9 +518,14 @@ cudaError_t lattice_fused_resident_fits(int kind, int threads, int Cp, size_t sm
     if (e != cudaSuccess) return e;
 #define GMRF_FR_FITS(KD, N, C)                                                                                  \
     if (kind == KD && threads == N && Cp == C) {                                                              \
-        e = allow_smem(lattice_fused_resident<KD, N, C>, smem);                                                \
+        int with_icpt = 0;                                                                                    \
+        e = allow_smem(lattice_fused_resident<KD, N, C, false>, smem);                                        \
+        if (e == cudaSuccess) e = allow_smem(lattice_fused_resident<KD, N, C, true>, smem);                   \
         if (e == cudaSuccess)                                                                                 \
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lattice_fused_resident<KD, N, C>, N, smem); \
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lattice_fused_resident<KD, N, C, false>, N, smem); \
+        if (e == cudaSuccess)                                                                                 \
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&with_icpt, lattice_fused_resident<KD, N, C, true>, N, smem); \
+        per_sm = per_sm < with_icpt ? per_sm : with_icpt;                                                     \
         if (e != cudaSuccess) {                                                                               \
             cudaGetLastError();                                                                               \
             return cudaSuccess; /* the shared memory does not fit: not resident */                            \
@@ -537,7 +552,9 @@ cudaError_t launch_lattice_fused_resident(int kind, int threads, int Cp, const T
     cfg.attrs = attr;
     cfg.numAttrs = 1;
 #define GMRF_FR_LAUNCH(KD, N, C) \
-    if (kind == KD && threads == N && Cp == C) return cudaLaunchKernelEx(&cfg, lattice_fused_resident<KD, N, C>, ra);
+    if (kind == KD && threads == N && Cp == C)                                                    \
+        return ra.h.draw_beta ? cudaLaunchKernelEx(&cfg, lattice_fused_resident<KD, N, C, true>, ra) \
+                              : cudaLaunchKernelEx(&cfg, lattice_fused_resident<KD, N, C, false>, ra);
     GMRF_FR_CONFIGS(GMRF_FR_LAUNCH)
 #undef GMRF_FR_LAUNCH
     return cudaErrorInvalidValue;
